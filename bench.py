@@ -774,7 +774,7 @@ def run_gpu(args):
                         "sample": "instances " + ",".join(map(str, sample)) + " (smallest of each level count, "
                                   "two of the three-level ones) against the FP64 oracle, relative L-inf over Omega_k"},
             "fp64": {"value": replica_rate(total, ms_64, world), "unit": "Mcells/s", "ms_per_step": ms_64},
-            "roofline": roofline("k_box_mid<df,16,*> (fused twiddle, local 16^3 FFTs, kernel product; one launch "
+            "roofline": roofline("k_line_mid<df,*> (z lines: forward transform, kernel product, inverse; one launch "
                                  "per box-mode level)", hb["alg_bytes"], mid_ms, hb["mid_launches"], pk,
                                  alg_flops=hb["alg_flops"],
                                  note="the kernel's time summed over the 64 instances run one by one with the "
@@ -782,7 +782,7 @@ def run_gpu(args):
                                       "work the kernel completes"),
             "roofline_solve": roofline("whole batched step", hb["alg_bytes"], ms_df, hb["launches"], pk,
                                        alg_flops=hb["alg_flops"], note="the step's graph time"),
-            "serial_phases_ms": {"k_box_mid": mid_ms, "block_index_dft_passes": hb["pas_ms"],
+            "serial_phases_ms": {"k_line_mid": mid_ms, "xy_line_passes": hb["pas_ms"],
                                  "all_solves_one_by_one": hb["serial_ms"]},
             "cpu_baseline": {"value": sample_cells / cpu_s / 1e6 if cpu_s else None, "unit": "Mcells/s",
                              "cores": os.cpu_count(), "kind": "oracle",

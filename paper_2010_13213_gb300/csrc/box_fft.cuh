@@ -3,15 +3,15 @@
 // A pass along one axis maps, per line and local cell, the nb inputs of the zero-padded length P = 2 nb
 // (forward) to its P outputs, or the P inputs back to the nb box outputs (inverse).  Splitting the outputs
 // (inputs) by parity turns both into two nb-point DFTs (Sec. 2.2's convolution; the block-index form of
-// box.cuh):
+// box_pass.cuh):
 //     forward  X_{2q} = DFT_nb(x)_q,            X_{2q+1} = DFT_nb(x_j W_P^j)_q,
 //     inverse  y_j = IDFT_nb(X_even)_j + W_P^{-j} IDFT_nb(X_odd)_j,
 // and each nb-point DFT runs as a mixed-radix Cooley-Tukey FFT over registers (radix 4, 2, 3, 5, 7; primes
 // 11 and 13 directly by conjugate pairs), every index a compile-time constant.  For nb = 16 a pass then
-// costs about a third of the direct conjugate-pair sums of box.cuh, whose work grows as nb^2.
+// costs about a third of the direct conjugate-pair sums of box_pass.cuh, whose work grows as nb^2.
 // Twiddles W_N^m (N | P) are read from the pass's parameter table W_P^{m P / N}.
 #pragma once
-#include "box.cuh"
+#include "box_pass.cuh"
 
 namespace lgf {
 
@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(NT) k_bfft_fwd(const cx<R> *__restrict__ in, c
       const int64_t e = (int64_t)idx * B3 + m;
       if (q.mask && !(q.mask[e] & q.bits)) return;
       const R v = load_field<R>(q.src, e, q.dtype);
-      if (q.part) im = im + v;
-      else re = re + v;
+      if (q.part != 0) im = im + v;
+      if (q.part != 1) re = re + v;
     };
     if (ns > 0) add(s0, 0);
     if (ns > 1) add(s1, 1);

@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(TC_ROWS) k_bdft_tc(const cx<R> *__restrict__ i
         const int64_t e = (int64_t)idx * B3 + m;
         if (q.mask && !(q.mask[e] & q.bits)) return;
         const R v = load_field<R>(q.src, e, q.dtype);
-        if (q.part) im = im + v;
-        else re = re + v;
+        if (q.part != 0) im = im + v;
+        if (q.part != 1) re = re + v;
       };
       if (ns > 0) add(s0);
       if (ns > 1) add(s1);

@@ -19,12 +19,43 @@ struct df {
   float hi, lo;
 };
 
+// v as hi + lo, hi the nearest float, lo the nearest float to the rest.  Within the floats' normal range by
+// integer and FP32 operations: the FP64 pipe (2 lanes a clock and SM; conversions to and from 64 bits run there
+// too) made the four FP64 instructions of the plain form a third of an x pass on the 96 x 96 x 48 ring.
 LGF_D df df_make(double v) {
+  const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v);
+  const unsigned e = (hw >> 20) & 0x7ffu;
+  if (e - 926u < 223u) {  // 2^-97 <= |v| < 2^126
+    // truncated to 24 bits: sign, exponent e - 896 (bit 7 of e flipped, the two bits above dropped), 23 bits
+    const unsigned tr = ((__funnelshift_l(lw, hw, 3) & 0x7fffffffu) ^ 0x40000000u) | (hw & 0x80000000u);
+    const unsigned rem = lw & 0x1fffffffu, up = rem >> 28;  // rest in 2^-29 ulp; round up from half an ulp
+    // rest / ulp - up: 15 bits / 2^15 (exact) plus 14 bits / 2^29 (exact), one rounding
+    const float a = __fsub_rn(__uint_as_float(0x3f800000u | ((rem >> 14) << 8)), __uint_as_float(0x3f800000u + (up << 23)));
+    const float b = __fsub_rn(__uint_as_float(0x38000000u | ((rem & 0x3fffu) << 9)), __uint_as_float(0x38000000u));
+    const float r = __fmul_rn(__fadd_rn(a, b), 1.1920928955078125e-7f);  // 2^-23
+    return {__uint_as_float(tr + up), __fmul_rn(r, __uint_as_float(tr & 0xff800000u))};
+  }
+  if (e <= 872u) return {__uint_as_float(hw & 0x80000000u), __uint_as_float(hw & 0x80000000u)};  // |v| < 2^-150: 0
   float h = __double2float_rn(v);
   float l = __double2float_rn(v - (double)h);
   return {h, l};
 }
-LGF_D double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
+// hi + lo in double: within 2^-100 <= |hi| < 2^127 the low part, rounded to hi's 2^-29 ulp, is added to hi's bit
+// pattern (no FP64 instruction, see df_make); |lo| <= ulp(hi) (a renormalised value).
+LGF_D double df_to_double(df a) {
+  const unsigned hb = __float_as_uint(a.hi), e = (hb >> 23) & 0xffu;
+  const float rel = __fmul_rn(a.lo, __uint_as_float((254u - e) << 23));  // lo / 2^exponent(hi)
+  if (e - 27u < 227u && fabsf(rel) <= 1.1920928955078125e-7f) {          // 2^-23
+    int q = __float2int_rn(__fmul_rn(rel, 4503599627370496.0f));         // 2^52
+    q = (hb >> 31) ? -q : q;                                             // towards (+) or away from hi's magnitude
+    if (q < 0 && !(hb & 0x7fffffu)) q *= 2;                              // below a power of two the ulp halves
+    const unsigned lw = hb << 29, hw = (((hb & 0x7fffffffu) >> 3) + 0x38000000u) | (hb & 0x80000000u);
+    const long long bits = (long long)(((unsigned long long)hw << 32) | lw) + (long long)q;
+    return __longlong_as_double(bits);
+  }
+  if (((hb << 1) | __float_as_uint(a.lo) << 1) == 0) return __hiloint2double((int)hb, 0);
+  return (double)a.hi + (double)a.lo;
+}
 
 LGF_D df df_add(df a, df b) {
   float s = __fadd_rn(a.hi, b.hi);

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/lgf.h"
+#include "arith.cuh"
 #include "common.cuh"
 
 namespace lgf {
@@ -105,19 +106,34 @@ struct TcMat {
 
 struct BoxSpec {
   int nb[3] = {0, 0, 0};
-  double *g64 = nullptr;  // [P^3 blocks][B^3] real spectrum, FP64
+  // real spectrum Ghat on 0 <= f_a <= L_a / 2, L_a = 2 nb_a B (even in every axis), x fastest
+  double *gf64 = nullptr;
+  float *gf32 = nullptr;
+  df *gfdf = nullptr;
+  // twiddles of the line transforms (lines.cuh): per-axis parameter tables, and W_{L_a}^n, n < L_a, on the device
+  // at entry ltl_off[a]
+  LineTw<double> lt64[3];
+  LineTw<float> lt32[3];
+  LineTw<df> ltdf[3];
+  Ar<double>::T *ltl64 = nullptr;
+  Ar<float>::T *ltl32 = nullptr;
+  Ar<df>::T *ltldf = nullptr;
+  int ltl_off[3] = {0, 0, 0};
+  int32_t *fx = nullptr;  // x frequency per row element: complex fields (2 nb_x B of them), then real fields
+  // the tensor-core DFT-GEMM (box_tc.cuh), the FP32 passes of box_pass.cuh and k_box_mid, built on the first solve that
+  // uses one of them: the spectrum in
+  // block order [P^3 blocks][B^3], the coefficient digits, and the four-step twiddles W_L^n, n < L = lcm(Pcx, Pcy,
+  // Pcz) (Pc = P B cells per axis; the twiddle of a cell m and block frequency K1 is
+  // W_L^{(sum_a m_a K1_a L / Pc_a) mod L})
+  bool blocks_ready = false;
+  cx<float> bw32[3][32];    // W_P^n per axis, n < P (host copies for kernel parameters)
   float *g32 = nullptr;
   df *gdf = nullptr;
-  // four-step twiddles: W_L^n, n < L = lcm(Pcx, Pcy, Pcz) (Pc = P B cells per axis); the twiddle of a
-  // cell m and block frequency K1 is W_L^{(sum_a m_a K1_a L / Pc_a) mod L}
   cx<double> *twl64 = nullptr;
   cx<float> *twl32 = nullptr;
   cx<df> *twldf = nullptr;
   int twL = 0;
   int twf[3] = {0, 0, 0};  // L / Pc_a
-  cx<double> bw64[3][32];  // W_P^n per axis, n < P (host copies for kernel parameters)
-  cx<float> bw32[3][32];
-  cx<df> bwdf[3][32];
   uint16_t *tcw = nullptr;  // device storage of the tensor-core coefficient digits
   TcMat tcm[3][3];          // per axis: forward, inverse, Hermitian-folded real inverse (axis 0 only)
   size_t bytes = 0;
@@ -160,7 +176,17 @@ struct Workspace {
 }  // namespace lgf
 
 namespace lgf {
-int box_spectrum(lgf_table *t, const int nb[3], BoxSpec **out, cudaStream_t st);
+// FP32 arithmetic on FP64 fields runs the block-index passes (box_pass.cuh says why).
+inline bool box_blocks(const lgf_solve_opts &o, int dtype) { return o.precision == LGF_PREC_FP32 && dtype == LGF_F64; }
+// The spectrum and tables of a box shape, built on first use; `blocks`: with those of the block-index paths.
+int box_spectrum(lgf_table *t, const int nb[3], bool blocks, BoxSpec **out, cudaStream_t st);
+// Bytes of the two scratch arrays of BoxOps::convolve for `nf` complex fields of `csize` bytes a value on `cells`
+// box cells: the line passes hold the x-transformed and the x- and y-transformed fields (2 and 4 values a cell),
+// the block-index passes the whole padded box twice.
+inline void box_scratch(int64_t nf, int64_t cells, size_t csize, bool blocks, size_t bytes[2]) {
+  bytes[0] = (size_t)nf * cells * csize * (blocks ? 8 : 2);
+  bytes[1] = (size_t)nf * cells * csize * (blocks ? 8 : 4);
+}
 // Synchronous read of the table's device status word; LGF_E_TIMEOUT (and the word cleared) when a
 // bounded device-side wait gave up since the last read.
 int take_device_status(lgf_table *t);

@@ -1,0 +1,6 @@
+// Line transforms of 16 points per second step, NB = 1..6, arithmetic double.
+#include "line_ops.cuh"
+
+namespace lgf {
+LINE_RANGE_DEFINE(double, 16, 1, 6, 1)
+}  // namespace lgf

@@ -188,7 +188,7 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
                         pair_cost(B, (double)L.SB.size(), (double)L.Tphi.size());
       use_box[k] = cb < cp;
     }
-    if (use_box[k]) maxbox = std::max<int64_t>(maxbox, (int64_t)std::min(ncomp, BOX_MAXF) * 8 * L.nbox * B3);
+    if (use_box[k]) maxbox = std::max<int64_t>(maxbox, L.nbox * B3);
   }
   for (int k = 0; k < K; ++k)
     if (!use_box[k] && !P->L[k].Tall.empty() && (o.mac_mode == LGF_MAC_BOX || !Gh))
@@ -197,9 +197,10 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
                        Gh ? "box support for it" : "pair spectra of this precision");
   Workspace *ws = workspace_for(t, st);
   const size_t field = sizeof(R) * (size_t)ncomp * maxBL * B3;
-  const size_t ybytes = sizeof(cx<R>) * (size_t)maxbox;
-  if ((rc = ws->buf[0].reserve(std::max(ybytes, sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSA, 1) * W))) ||
-      (rc = ws->buf[1].reserve(std::max(ybytes, sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxT, 1) * W))) ||
+  size_t ybytes[2];
+  box_scratch(std::min(ncomp, BOX_MAXF), maxbox, sizeof(cx<R>), o.dft_slices > 0 || box_blocks(o, dtype), ybytes);
+  if ((rc = ws->buf[0].reserve(std::max(ybytes[0], sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSA, 1) * W))) ||
+      (rc = ws->buf[1].reserve(std::max(ybytes[1], sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxT, 1) * W))) ||
       (rc = ws->buf[3].reserve(sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSB, 1) * W)) ||
       (rc = ws->buf[4].reserve(sizeof(R) * (size_t)Foff[K])) || (rc = ws->buf[5].reserve(field)) ||
       (rc = ws->buf[6].reserve(field)) || (rc = ws->buf[7].reserve(sizeof(R) * (size_t)Foff[K])) ||
@@ -271,10 +272,10 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
     }
     if (use_box[k]) {
       BoxSpec *S = nullptr;
-      if ((rc = box_spectrum(t, L.box_nb, &S, st))) return rc;
+      if ((rc = box_spectrum(t, L.box_nb, o.dft_slices > 0 || box_blocks(o, dtype), &S, st))) return rc;
       const int32_t *gA = L.d_box, *gB = gA + L.nbox, *sPsi = gB + L.nbox, *sPhi = sPsi + L.nbox;
       const double hk = m->h0 / (double)(1 << k);
-      const double scale = hk * hk / (8.0 * L.nbox * (double)B3);
+      const double scale = hk * hk;
       const bool packAB = nPsi > 0 || nSB > 0;
       const R *cadd = k > 0 ? c : nullptr;
       cx<R> *Y0 = (cx<R> *)ws->buf[0].p, *Y1 = (cx<R> *)ws->buf[1].p;
@@ -286,10 +287,7 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
         for (int cc = 0; cc < ncomp; ++cc) {
           InSpec sp[3];
           int ns = 0;
-          if (nSA) {
-            sp[ns++] = InSpec{gA, A + cc * cs[k], nullptr, 2, 0, 0};
-            sp[ns++] = InSpec{gA, A + cc * cs[k], nullptr, 2, 0, 1};
-          }
+          if (nSA) sp[ns++] = InSpec{gA, A + cc * cs[k], nullptr, 2, 0, 2};
           if (nSB) sp[ns++] = InSpec{gB, Fall + Foff[k] + cc * cs[k], L.d_cellmask, 2, CB_COV, 1};
           nin.push_back(ns);
           in.emplace_back();
@@ -319,7 +317,8 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
       }
       const int nf = (int)nin.size();
       if ((rc = BoxOps<R>::convolve(B, S, nf, nin.data(), in.data(), ore.data(), oim.data(), scale, Y0, Y1, st,
-                                    o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, t->d_status, &launches)))
+                                    o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, box_blocks(o, dtype),
+                                    t->d_status, &launches)))
         return rc;
       target_cells += L.n_omega;
       nsrc_total += nSA + nSB;

@@ -257,18 +257,19 @@ static int solve_single_box(lgf_table *t, const lgf_mesh *m, const SinglePlan *P
   const int B = m->block, n = m->nblocks[0];
   const int64_t B3 = (int64_t)B * B * B;
   BoxSpec *S = nullptr;
-  int rc = box_spectrum(t, P->nb, &S, st);
+  int rc = box_spectrum(t, P->nb, o.dft_slices > 0 || box_blocks(o, dtype), &S, st);
   if (rc) return rc;
   Workspace *ws = workspace_for(t, st);
   const int nf = (ncomp + 1) / 2;
-  const size_t ybytes = sizeof(cx<R>) * (size_t)std::min(nf, BOX_MAXF) * (8 * P->nbox) * B3;
-  if ((rc = ws->buf[0].reserve(ybytes)) || (rc = ws->buf[1].reserve(ybytes))) return rc;
+  size_t ybytes[2];
+  box_scratch(std::min(nf, BOX_MAXF), P->nbox * B3, sizeof(cx<R>), o.dft_slices > 0 || box_blocks(o, dtype), ybytes);
+  if ((rc = ws->buf[0].reserve(ybytes[0])) || (rc = ws->buf[1].reserve(ybytes[1]))) return rc;
   const int32_t *gmap = P->d_idx + P->nsrc + P->ntgt, *smap = gmap + P->nbox;
   PhaseTimer tm;
   tm.start(o.timing != 0, st);
   const int64_t cs = (int64_t)n * B3;
   const size_t es = dtype_size(dtype, sizeof(R));
-  const double scale = m->h0 * m->h0 / (8.0 * P->nbox * (double)B3);
+  const double scale = m->h0 * m->h0;
   // two components per complex field
   std::vector<int> nin(nf);
   std::vector<InSpec3> in(nf);
@@ -284,7 +285,8 @@ static int solve_single_box(lgf_table *t, const lgf_mesh *m, const SinglePlan *P
   int64_t launches = 0;
   if ((rc = BoxOps<R>::convolve(B, S, nf, nin.data(), in.data(), ore.data(), oim.data(), scale,
                                 (cx<R> *)ws->buf[0].p, (cx<R> *)ws->buf[1].p, st,
-                                o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, t->d_status, &launches)))
+                                o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, box_blocks(o, dtype),
+                                t->d_status, &launches)))
     return rc;
   tm.finish(rep);
   fill_report(rep, P, B3, ws, launches, LGF_MAC_BOX, (int64_t)S->bytes);
