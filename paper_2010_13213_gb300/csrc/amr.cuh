@@ -10,7 +10,7 @@
 // Fields are stored per level as [ncomp][nBL][B^3] over the level's internal block set; a dense
 // block map (block coords -> index, -1 if absent) gives neighbours across block boundaries.
 #pragma once
-#include "common.cuh"
+#include "arith.cuh"
 
 struct LevelDev {
   const int32_t *map;      // [n.z][n.y][n.x] block map
@@ -487,6 +487,126 @@ __global__ void __launch_bounds__(B * B) k_heat_line(LevelDev L, const int4 *blo
 }
 template <class R, int B>
 size_t heat_line_smem(int r) { return sizeof(R) * (size_t)(B + 2 * r) * (B * B + 1); }
+
+// The same pass in double-float with packed arithmetic: a thread sums a pair of adjacent lines (q = 2p, 2p + 1) as
+// f32x2 chains on (hi, hi) and (lo, lo) register pairs, the same operations as the scalar form and the same results.
+// The tile holds S[t][p] = (hi_2p, hi_2p+1, lo_2p, lo_2p+1).  Along y and z the pair is two neighbours in x: a thread
+// loads, sums and stores its own column (16-byte accesses); along x the tile is filled and read back in memory order.
+// Bound: the FP32 pipe (10 (2 r + 1) packed instructions per output; the scalar form issues twice as many and spent a
+// third of its issue slots on the index arithmetic of the staging) and, with three CTAs per SM for the tiles, the
+// latency of the staging.  The nine passes of the three-level ring (r = 6, 8, 10): 725 us; reading both taps of every
+// pair from the tile instead of the two windows 760 us.
+// grid (|HB|, ncomp), B^2 / 2 threads, (B + 2 r)(B^2 / 2 + 1) 16-byte values of dynamic shared memory.
+template <int B>
+__global__ void __launch_bounds__(B * B / 2) k_heat_pair(LevelDev L, const int4 *blocks, const int32_t *HB, int axis,
+                                                         const df *in, df *out, int64_t cs, HeatW w) {
+  using namespace lgf;
+  constexpr int B2 = B * B, B3 = B * B2, NT = B2 / 2, PS = NT + 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  ulonglong2 *S = reinterpret_cast<ulonglong2 *>(smem_raw);
+  __shared__ f2 wh[B + 1], wl[B + 1];
+  const int r = w.r, p = threadIdx.x;
+  const int b = HB[blockIdx.x], comp = blockIdx.y;
+  const int4 bc = blocks[b];
+  for (int d = p; d <= r; d += NT) {
+    const df v = RT<df>::from(w.w[d]);
+    wh[d] = f2_pack(v.hi, v.hi);
+    wl[d] = f2_pack(v.lo, v.lo);
+  }
+  const int nbm = level_block(L, bc.x - (axis == 0), bc.y - (axis == 1), bc.z - (axis == 2));
+  const int nbp = level_block(L, bc.x + (axis == 0), bc.y + (axis == 1), bc.z + (axis == 2));
+  const df *src = in + comp * cs;
+  const int step = axis == 1 ? B : B2;  // elements per cell along y or z
+  const int col = axis == 1 ? (p % (B / 2)) * 2 + (p / (B / 2)) * B2 : 2 * p;
+  const int T = B + 2 * r;
+  if (axis != 0) {
+#pragma unroll 4
+    for (int t = 0; t < T; ++t) {
+      const int la = t - r, blk = la < 0 ? nbm : (la >= B ? nbp : b);
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (blk >= 0) v = *reinterpret_cast<const float4 *>(src + (int64_t)blk * B3 + col + (la & (B - 1)) * step);
+      S[t * PS + p] = make_ulonglong2(f2_pack(v.x, v.z), f2_pack(v.y, v.w));
+    }
+  } else {
+    // B lanes per line: element (t, q) goes to float (q & 1) of the high and of the low pair
+    float *F = reinterpret_cast<float *>(S);
+    const int x = p % B;
+    auto put = [&](int t, int q, int blk, int cell) {
+      df v{0.0f, 0.0f};
+      if (blk >= 0) v = src[(int64_t)blk * B3 + q * B + cell];
+      float *o = F + (t * PS + (q >> 1)) * 4 + (q & 1);
+      o[0] = v.hi;
+      o[2] = v.lo;
+    };
+#pragma unroll 4
+    for (int q = p / B; q < B2; q += NT / B) {
+      put(r + x, q, b, x);
+      if (x < r) {
+        put(x, q, nbm, B - r + x);
+        put(r + B + x, q, nbp, x);
+      }
+    }
+  }
+  __syncthreads();
+  typedef Ar<df> A;
+  // eight outputs at a time; the values d cells above and below them sit in two rotating windows, so that a tap loads
+  // one new value per window instead of eight
+  const f2 w0h = wh[0], w0l = wl[0];
+  df *dst = out + comp * cs + (int64_t)b * B3;
+#pragma unroll 1
+  for (int t0 = 0; t0 < B; t0 += 8) {
+    const ulonglong2 *C = S + (t0 + r) * PS + p;
+    A::V acc[8], up[8], dn[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = A::norm(A::mulr(A::ld(C + i * PS), w0h, w0l));
+    if (r > 0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) up[i] = A::ld(C + (i + 1) * PS), dn[i] = A::ld(C + (i - 1) * PS);
+    }
+#pragma unroll 1
+    for (int d0 = 0; d0 < r; d0 += 8) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int d = d0 + k + 1;  // up[(i + k) & 7] is cell i + d, dn[(i - k) & 7] cell i - d
+        if (d > r) break;
+        const f2 h = wh[d], l = wl[d];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const A::V x = A::add(up[(i + k) & 7], dn[(i - k) & 7]);
+          const f2 q = f2_mul(x.h, h);
+          f2 e = f2_fma(x.h, h, f2_neg(q));
+          e = f2_fma(x.h, l, e);
+          acc[i] = A::add(acc[i], A::V{q, f2_fma(x.l, h, e)});
+        }
+        if (d < r) up[k] = A::ld(C + (8 + d) * PS), dn[(7 - k) & 7] = A::ld(C + (-1 - d) * PS);
+      }
+    }
+    if (axis != 0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const A::V v = A::norm(acc[i]);
+        float4 o;
+        f2_unpack(v.h, o.x, o.z);
+        f2_unpack(v.l, o.y, o.w);
+        *reinterpret_cast<float4 *>(dst + col + (t0 + i) * step) = o;
+      }
+    } else {  // rows t0 .. t0 + 7: the later outputs of the column read rows from t0 + 8 on
+#pragma unroll
+      for (int i = 0; i < 8; ++i) A::st(S + (t0 + i) * PS + p, A::norm(acc[i]));
+    }
+  }
+  if (axis != 0) return;
+  __syncthreads();
+  const float *F = reinterpret_cast<const float *>(S);
+  const int x = p % B;
+#pragma unroll 4
+  for (int q = p / B; q < B2; q += NT / B) {
+    const float *o = F + (x * PS + (q >> 1)) * 4 + (q & 1);
+    dst[q * B + x] = df{o[0], o[2]};
+  }
+}
+template <int B>
+size_t heat_pair_smem(int r) { return sizeof(ulonglong2) * (size_t)(B + 2 * r) * (B * B / 2 + 1); }
 
 // The same pass for radii r > B: every tap looks its cell up in the block map; absent cells read 0.
 template <class R>

@@ -526,12 +526,20 @@ template <class R, int BB>
 static int heat_line_launch(const LevelDev &Ld, const int4 *BL, const int32_t *HB, int nHB, int ncomp, int ax,
                             const R *in, R *out, int64_t cs, const HeatW &w, cudaStream_t st) {
   static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_heat_line<R, BB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)heat_line_smem<R, BB>(BB));
-    attr = true;
+  if constexpr (std::is_same<R, df>::value) {
+    if (!attr) {
+      cudaFuncSetAttribute(k_heat_pair<BB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)heat_pair_smem<BB>(BB));
+      attr = true;
+    }
+    k_heat_pair<BB><<<dim3(nHB, ncomp), BB * BB / 2, heat_pair_smem<BB>(w.r), st>>>(Ld, BL, HB, ax, in, out, cs, w);
+  } else {
+    if (!attr) {
+      cudaFuncSetAttribute(k_heat_line<R, BB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)heat_line_smem<R, BB>(BB));
+      attr = true;
+    }
+    k_heat_line<R, BB><<<dim3(nHB, ncomp), BB * BB, heat_line_smem<R, BB>(w.r), st>>>(Ld, BL, HB, ax, in, out, cs, w);
   }
-  k_heat_line<R, BB><<<dim3(nHB, ncomp), BB * BB, heat_line_smem<R, BB>(w.r), st>>>(Ld, BL, HB, ax, in, out, cs, w);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LGF_OK : set_error(LGF_E_CUDA, "heat pass launch: %s", cudaGetErrorString(e));
 }
@@ -598,11 +606,9 @@ static int heat_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, voi
     const LevelDev Lc = k > 0 ? level_dev(P, k - 1, m->h0) : Ld;
     const int nHB = (int)L.HB.size();
     const int32_t *HB = L.d_lists + L.off_HB;
-    const size_t bytes = sizeof(R) * (size_t)ncomp * L.BL.size() * B3;
-    cudaMemsetAsync(T0, 0, bytes, st);
-    cudaMemsetAsync(T1, 0, bytes, st);
-    cudaMemsetAsync(Ucur, 0, bytes, st);
-    // P_k fhat into Ucur: the heat passes' source, kept for the next level's interpolation
+    // P_k fhat into Ucur: the heat passes' source, kept for the next level's interpolation.  The buffers are not
+    // cleared: every cell that a result reads (Omega_k within the kernel radius, and the next level's interpolation
+    // stencils) lies in the heat block set, which the reconstruction and each pass write whole.
     k_heat_build<R><<<dim3(nHB, ncomp), 256, sizeof(R) * (size_t)interp_sep_values(B), st>>>(
         Ld, L.d_BL, HB, Fall + Foff[k], L.nU, Ucur, cs[k], Lc, Uprev, k > 0 ? cs[k - 1] : 0, k > 0);
     LGF_LAUNCH_CHECK("heat source");
@@ -721,8 +727,6 @@ static int reconstruct_levels(Plan *P, const lgf_mesh *m, int ncomp, const void 
     const LevelDev Lc = k > 0 ? level_dev(P, k - 1, m->h0) : Ld;
     const int nHB = (int)L.HB.size();
     const int32_t *HB = L.d_lists + L.off_HB;
-    const size_t bytes = sizeof(R) * (size_t)ncomp * L.BL.size() * B3;
-    cudaMemsetAsync(Ucur, 0, bytes, st);
     k_heat_build<R><<<dim3(nHB, ncomp), 256, sizeof(R) * (size_t)interp_sep_values(B), st>>>(
         Ld, L.d_BL, HB, Fall + Foff[k], L.nU, Ucur, cs[k], Lc, Uprev, k > 0 ? cs[k - 1] : 0, k > 0);
     LGF_LAUNCH_CHECK("reconstruction");
