@@ -650,16 +650,21 @@ __global__ void __launch_bounds__(256) k_proj_div(LevelDev L, const int4 *blocks
   const int b = blockIdx.x, sh = L.shift, B = 1 << sh, B3 = B * B * B;
   const int4 bc = blocks[b];
   const double inv_h = 1.0 / L.h;
+  // the blocks below along each axis, looked up once
+  const int nx = level_block(L, bc.x - 1, bc.y, bc.z), ny = level_block(L, bc.x, bc.y - 1, bc.z),
+            nz = level_block(L, bc.x, bc.y, bc.z - 1);
+  // component a of the cell one step toward -e_a: this block, or the last layer of the one below (NaN when absent)
+  auto below = [&](int a, int nb, int off, int c, int st) -> double {
+    if (c > 0) return RT<R>::to_d(T[a * cs + (int64_t)b * B3 + off - st]);
+    return nb < 0 ? nan("") : RT<R>::to_d(T[a * cs + (int64_t)nb * B3 + off + (B - 1) * st]);
+  };
   for (int off = threadIdx.x; off < B3; off += blockDim.x) {
     double d = 0.0;
     if (L.cellmask[(int64_t)b * B3 + off] & 1) {
-      const int x = (bc.x << sh) + (off & (B - 1)), y = (bc.y << sh) + ((off >> sh) & (B - 1)),
-                z = (bc.z << sh) + (off >> (2 * sh));
       const double here = RT<R>::to_d(T[(int64_t)b * B3 + off]) + RT<R>::to_d(T[cs + (int64_t)b * B3 + off]) +
                           RT<R>::to_d(T[2 * cs + (int64_t)b * B3 + off]);
-      const double back = RT<R>::to_d(fetch<R>(L, T, cs, 0, x - 1, y, z)) +
-                          RT<R>::to_d(fetch<R>(L, T, cs, 1, x, y - 1, z)) +
-                          RT<R>::to_d(fetch<R>(L, T, cs, 2, x, y, z - 1));
+      const double back = below(0, nx, off, off & (B - 1), 1) + below(1, ny, off, (off >> sh) & (B - 1), B) +
+                          below(2, nz, off, off >> (2 * sh), B * B);
       d = (here - back) * inv_h;
     }
     store_field(out, (user_off + b) * (int64_t)B3 + off, dtype, d);
@@ -675,13 +680,15 @@ __global__ void __launch_bounds__(256) k_proj_grad(LevelDev L, const int4 *block
   const int4 bc = blocks[b];
   const double inv_h = 1.0 / L.h;
   const int64_t o0 = a * ucs + (user_off + b) * (int64_t)B3;
+  const int nb = level_block(L, bc.x + (a == 0), bc.y + (a == 1), bc.z + (a == 2));  // the block above along axis a
+  const int st = 1 << (a * sh);
   for (int off = threadIdx.x; off < B3; off += blockDim.x) {
     double v = 0.0;
     if (L.cellmask[(int64_t)b * B3 + off] & 1) {
-      const int x = (bc.x << sh) + (off & (B - 1)), y = (bc.y << sh) + ((off >> sh) & (B - 1)),
-                z = (bc.z << sh) + (off >> (2 * sh));
+      const int c = (off >> (a * sh)) & (B - 1);
       const double pn = RT<R>::to_d(T[(int64_t)b * B3 + off]);
-      const double pe = RT<R>::to_d(fetch<R>(L, T, cs, 0, x + (a == 0), y + (a == 1), z + (a == 2)));
+      const double pe = c < B - 1 ? RT<R>::to_d(T[(int64_t)b * B3 + off + st])
+                                  : (nb < 0 ? nan("") : RT<R>::to_d(T[(int64_t)nb * B3 + off - (B - 1) * st]));
       v = load_field<double>(r, o0 + off, dtype) - (pe - pn) * inv_h;
     }
     store_field(w, o0 + off, dtype, v);
