@@ -224,8 +224,8 @@ int lgf_heat_apply(lgf_table *t, const lgf_mesh *m, int32_t ncomp, const void *f
  *   u_dev        : device [3][nblocks][B^3] in dtype; every cell written.
  *   opts, rep    : as for lgf_poisson_solve (the report is the streamfunction solve's, with the curl
  *                  kernel added to kernel_launches).
- * Scratch: the vorticity and the streamfunction on the extended block set, allocated and freed in
- * stream order.  Errors: as lgf_poisson_solve; LGF_E_MESH for nlevels != 1; LGF_E_OOM for the scratch.
+ * Scratch: the vorticity and the streamfunction on the extended block set, held by the table per stream.
+ * Errors: as lgf_poisson_solve; LGF_E_MESH for nlevels != 1; LGF_E_OOM for the scratch.
  */
 int lgf_velocity_refresh(lgf_table *t, const lgf_mesh *m, const void *omega_dev, void *u_dev, int32_t dtype,
                          const lgf_solve_opts *opts, lgf_report *rep, void *cuda_stream);

@@ -12,7 +12,11 @@
 #include <cuda_runtime.h>
 #include <string.h>
 
+#include <list>
 #include <map>
+#include <memory>
+#include <mutex>
+#include <string>
 #include <tuple>
 #include <vector>
 
@@ -48,6 +52,64 @@ __global__ void __launch_bounds__(256) k_curl_t(const T *__restrict__ psi, int64
   }
 }
 
+// Extended block set of a mesh (the caller's blocks first, then their missing -x, -y, -z neighbours as targets only)
+// and the neighbour table on the device, cached by geometry as the solver's plans are.
+struct RefreshPlan {
+  std::vector<int32_t> ijk;
+  std::vector<uint8_t> roles;
+  int32_t *d_nbr = nullptr;
+  int next = 0;
+  ~RefreshPlan() { cudaFree(d_nbr); }
+};
+static std::mutex g_rp_mu;
+static std::list<std::pair<std::string, std::shared_ptr<RefreshPlan>>> g_rp;  // most recent first
+
+static int refresh_plan(const lgf_mesh *m, std::shared_ptr<RefreshPlan> &out) {
+  const int n = m->nblocks[0];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::string key((const char *)&dev, sizeof dev);
+  key.append((const char *)&m->block, 4);
+  key.append((const char *)m->block_ijk, 12 * (size_t)n);
+  std::lock_guard<std::mutex> g(g_rp_mu);
+  for (auto it = g_rp.begin(); it != g_rp.end(); ++it)
+    if (it->first == key) {
+      g_rp.splice(g_rp.begin(), g_rp, it);
+      out = it->second;
+      return LGF_OK;
+    }
+  auto P = std::make_shared<RefreshPlan>();
+  std::map<std::tuple<int, int, int>, int> index;
+  P->ijk.assign(m->block_ijk, m->block_ijk + 3 * (size_t)n);
+  for (int i = 0; i < n; ++i) index[std::make_tuple(P->ijk[3 * i], P->ijk[3 * i + 1], P->ijk[3 * i + 2])] = i;
+  std::vector<int32_t> nbr(3 * (size_t)n);
+  for (int i = 0; i < n; ++i)
+    for (int a = 0; a < 3; ++a) {
+      int c[3] = {m->block_ijk[3 * i], m->block_ijk[3 * i + 1], m->block_ijk[3 * i + 2]};
+      --c[a];
+      const auto at = std::make_tuple(c[0], c[1], c[2]);
+      auto it = index.find(at);
+      if (it == index.end()) {
+        it = index.emplace(at, (int)(P->ijk.size() / 3)).first;
+        P->ijk.insert(P->ijk.end(), c, c + 3);
+      }
+      nbr[3 * i + a] = it->second;
+    }
+  P->next = (int)(P->ijk.size() / 3);
+  P->roles.assign(P->next, 2);
+  for (int i = 0; i < n; ++i) P->roles[i] = 3;
+  if (cudaMalloc(&P->d_nbr, sizeof(int32_t) * nbr.size()) != cudaSuccess) {
+    cudaGetLastError();
+    return set_error(LGF_E_OOM, "velocity refresh neighbour table");
+  }
+  if (cudaMemcpy(P->d_nbr, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+    return set_error(LGF_E_CUDA, "velocity refresh neighbour table upload");
+  g_rp.emplace_front(key, P);
+  while (g_rp.size() > 1024) g_rp.pop_back();  // cudaFree inside orders against in-flight work
+  out = P;
+  return LGF_OK;
+}
+
 }  // namespace lgf
 
 using namespace lgf;
@@ -71,64 +133,36 @@ extern "C" int lgf_velocity_refresh(lgf_table *t, const lgf_mesh *m, const void 
   const int B = m->block, n = m->nblocks[0];
   const int shift = B == 8 ? 3 : 4;
   const int64_t B3 = (int64_t)B * B * B;
-  // extended block set: the caller's blocks first, then the missing -x, -y, -z neighbours
-  std::map<std::tuple<int, int, int>, int> index;
-  std::vector<int32_t> ijk(m->block_ijk, m->block_ijk + 3 * (size_t)n);
-  for (int i = 0; i < n; ++i) index[std::make_tuple(ijk[3 * i], ijk[3 * i + 1], ijk[3 * i + 2])] = i;
-  std::vector<int32_t> nbr(3 * (size_t)n);
-  for (int i = 0; i < n; ++i)
-    for (int a = 0; a < 3; ++a) {
-      int c[3] = {m->block_ijk[3 * i], m->block_ijk[3 * i + 1], m->block_ijk[3 * i + 2]};
-      --c[a];
-      const auto key = std::make_tuple(c[0], c[1], c[2]);
-      auto it = index.find(key);
-      if (it == index.end()) {
-        it = index.emplace(key, (int)(ijk.size() / 3)).first;
-        ijk.insert(ijk.end(), c, c + 3);
-      }
-      nbr[3 * i + a] = it->second;
-    }
-  const int next = (int)(ijk.size() / 3);
-  std::vector<uint8_t> roles(next, 2);  // added blocks: targets only
-  for (int i = 0; i < n; ++i) roles[i] = 3;
+  std::shared_ptr<RefreshPlan> P;
+  if ((rc = refresh_plan(m, P))) return rc;
+  const int next = P->next;
   lgf_mesh me = *m;
-  int32_t nb_ext[1] = {next};
+  const int32_t nb_ext[1] = {next};
   me.nblocks = nb_ext;
-  me.block_ijk = ijk.data();
-  me.block_role = roles.data();
-  // scratch (stream-ordered): omega on the extended set (the added blocks are not sources, never read),
-  // psi on the extended set, the neighbour table
+  me.block_ijk = P->ijk.data();
+  me.block_role = P->roles.data();
+  // scratch of the table's workspace for this stream: omega on the extended set (the added blocks are not sources,
+  // never read) and psi on the extended set
   const size_t es = dtype == LGF_F64 ? 8 : 4;
   const int64_t ext_cs = (int64_t)next * B3, ucs = (int64_t)n * B3;
-  void *om = nullptr, *psi = nullptr, *dnbr = nullptr;
-  if (cudaMallocAsync(&om, es * 3 * (size_t)ext_cs, st) != cudaSuccess ||
-      cudaMallocAsync(&psi, es * 3 * (size_t)ext_cs, st) != cudaSuccess ||
-      cudaMallocAsync(&dnbr, sizeof(int32_t) * nbr.size(), st) != cudaSuccess) {
-    if (om) cudaFreeAsync(om, st);
-    if (psi) cudaFreeAsync(psi, st);
-    if (dnbr) cudaFreeAsync(dnbr, st);
-    cudaGetLastError();
-    return set_error(LGF_E_OOM, "velocity refresh scratch (%zu bytes)", 2 * es * 3 * (size_t)ext_cs);
-  }
+  Workspace *ws = workspace_for(t, st);
+  if ((rc = ws->buf[21].reserve(es * 3 * (size_t)ext_cs)) || (rc = ws->buf[22].reserve(es * 3 * (size_t)ext_cs))) return rc;
+  void *om = ws->buf[21].p, *psi = ws->buf[22].p;
   for (int c = 0; c < 3; ++c)
     cudaMemcpyAsync((char *)om + es * c * ext_cs, (const char *)omega_dev + es * c * ucs, es * ucs,
                     cudaMemcpyDeviceToDevice, st);
-  cudaMemcpyAsync(dnbr, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice, st);
   rc = solve_poisson(t, &me, 3, om, psi, dtype, o, rep, st);
   if (rc == LGF_OK) {
     const double inv_h = 1.0 / m->h0;
     if (dtype == LGF_F64)
-      k_curl_t<double><<<dim3(n, 3), 256, 0, st>>>((const double *)psi, ext_cs, (const int32_t *)dnbr, shift, inv_h,
+      k_curl_t<double><<<dim3(n, 3), 256, 0, st>>>((const double *)psi, ext_cs, P->d_nbr, shift, inv_h,
                                                   (double *)u_dev, ucs);
     else
-      k_curl_t<float><<<dim3(n, 3), 256, 0, st>>>((const float *)psi, ext_cs, (const int32_t *)dnbr, shift, inv_h,
+      k_curl_t<float><<<dim3(n, 3), 256, 0, st>>>((const float *)psi, ext_cs, P->d_nbr, shift, inv_h,
                                                  (float *)u_dev, ucs);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) rc = set_error(LGF_E_CUDA, "curl launch: %s", cudaGetErrorString(e));
     else if (rep) rep->kernel_launches += 1;
   }
-  cudaFreeAsync(om, st);
-  cudaFreeAsync(psi, st);
-  cudaFreeAsync(dnbr, st);
   return rc;
 }
