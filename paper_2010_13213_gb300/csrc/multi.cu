@@ -642,8 +642,13 @@ static int heat_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, voi
 // Staggered fields: component a of a face field at cell n sits on the face n + (1/2,1/2,1/2) + e_a/2; the
 // pressure at the cell centre.  D r(n) = sum_a (r_a[n] - r_a[n - e_a]) / h, (G p)_a[n] = (p[n + e_a] - p[n]) / h.
 
+// CTAs per block of the divergence and the gradient: levels of about a hundred blocks leave most of the chip idle with
+// one CTA per block, each thread with a chain of sixteen cells (stage projection of the two-level ring 1,128 us with one,
+// 1,064 us with four).
+#define PROJ_PARTS 4
+
 // D^r on the Omega_k cells of the caller's level-k blocks from the reconstruction T = P_k r^ (3 components,
-// internal layout); 0 on the other cells.  grid (nU_k), 256 threads; out in the caller's layout (dtype).
+// internal layout); 0 on the other cells.  grid (nU_k, PROJ_PARTS), 256 threads; out in the caller's layout (dtype).
 template <class R>
 __global__ void __launch_bounds__(256) k_proj_div(LevelDev L, const int4 *blocks, const R *T, int64_t cs, void *out,
                                                   int dtype, int64_t user_off) {
@@ -658,7 +663,8 @@ __global__ void __launch_bounds__(256) k_proj_div(LevelDev L, const int4 *blocks
     if (c > 0) return RT<R>::to_d(T[a * cs + (int64_t)b * B3 + off - st]);
     return nb < 0 ? nan("") : RT<R>::to_d(T[a * cs + (int64_t)nb * B3 + off + (B - 1) * st]);
   };
-  for (int off = threadIdx.x; off < B3; off += blockDim.x) {
+  const int part = B3 / PROJ_PARTS, end = (blockIdx.y + 1) * part;
+  for (int off = blockIdx.y * part + threadIdx.x; off < end; off += blockDim.x) {
     double d = 0.0;
     if (L.cellmask[(int64_t)b * B3 + off] & 1) {
       const double here = RT<R>::to_d(T[(int64_t)b * B3 + off]) + RT<R>::to_d(T[cs + (int64_t)b * B3 + off]) +
@@ -672,7 +678,7 @@ __global__ void __launch_bounds__(256) k_proj_div(LevelDev L, const int4 *blocks
 }
 
 // w^ = r^ - G p on the Omega_k cells from the caller's r and the reconstruction T = P_k p^ (1 component); 0 on
-// the other cells.  grid (nU_k, 3).
+// the other cells.  grid (nU_k, 3, PROJ_PARTS).
 template <class R>
 __global__ void __launch_bounds__(256) k_proj_grad(LevelDev L, const int4 *blocks, const R *T, int64_t cs,
                                                    const void *r, void *w, int dtype, int64_t ucs, int64_t user_off) {
@@ -682,7 +688,8 @@ __global__ void __launch_bounds__(256) k_proj_grad(LevelDev L, const int4 *block
   const int64_t o0 = a * ucs + (user_off + b) * (int64_t)B3;
   const int nb = level_block(L, bc.x + (a == 0), bc.y + (a == 1), bc.z + (a == 2));  // the block above along axis a
   const int st = 1 << (a * sh);
-  for (int off = threadIdx.x; off < B3; off += blockDim.x) {
+  const int part = B3 / PROJ_PARTS, end = (blockIdx.z + 1) * part;
+  for (int off = blockIdx.z * part + threadIdx.x; off < end; off += blockDim.x) {
     double v = 0.0;
     if (L.cellmask[(int64_t)b * B3 + off] & 1) {
       const int c = (off >> (a * sh)) & (B - 1);
@@ -773,7 +780,7 @@ static int projection_t(lgf_table *t, const lgf_mesh *m_in, const void *r, void 
   rc = reconstruct_levels<R>(P, &m, 3, r, dtype, ws, launches, st,
                              [&](int k, const LevelDev &Ld, const R *T, int64_t cs) {
                                const LevelPlan &L = P->L[k];
-                               k_proj_div<R><<<L.nU, 256, 0, st>>>(Ld, L.d_BL, T, cs, d, dtype, L.user_off);
+                               k_proj_div<R><<<dim3(L.nU, PROJ_PARTS), 256, 0, st>>>(Ld, L.d_BL, T, cs, d, dtype, L.user_off);
                                cudaError_t e = cudaGetLastError();
                                return e == cudaSuccess ? LGF_OK
                                                        : set_error(LGF_E_CUDA, "divergence launch: %s",
@@ -793,7 +800,7 @@ static int projection_t(lgf_table *t, const lgf_mesh *m_in, const void *r, void 
   rc = reconstruct_levels<R>(P, &m, 1, p, dtype, ws, launches, st,
                              [&](int k, const LevelDev &Ld, const R *T, int64_t cs) {
                                const LevelPlan &L = P->L[k];
-                               k_proj_grad<R><<<dim3(L.nU, 3), 256, 0, st>>>(Ld, L.d_BL, T, cs, r, w, dtype, ucs,
+                               k_proj_grad<R><<<dim3(L.nU, 3, PROJ_PARTS), 256, 0, st>>>(Ld, L.d_BL, T, cs, r, w, dtype, ucs,
                                                                             L.user_off);
                                cudaError_t e = cudaGetLastError();
                                return e == cudaSuccess ? LGF_OK
