@@ -524,7 +524,7 @@ def heat_line(L, torch, dev, steps, warmup, world, pk, flush):
             "phases_ms": {"restrict": float(rep.ms_phase[0]), "build": float(rep.ms_phase[5]),
                           "passes_and_store": float(rep.ms_phase[7])},
             "gpu_launches": int(rep.kernel_launches),
-            "roofline": roofline("k_heat_line x 3 + k_heat_store (per level)", passes_bytes, rep.ms_phase[7],
+            "roofline": roofline("k_heat_pair x 3 + k_heat_store (per level)", passes_bytes, rep.ms_phase[7],
                                  4 * len(mesh["levels"]), pk,
                                  note="for the heat passes: 8 bytes in + 8 out per target cell-component and pass"),
             "e2e": {"value": cells / (e2e_ms * 1e-3) / 1e6, "unit": "Mcells/s",
