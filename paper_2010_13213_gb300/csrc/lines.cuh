@@ -44,14 +44,16 @@ namespace lgf {
 
 // Lines per CTA: enough (line, K1) tasks for the 128 threads with small NB, shared memory for three or four CTAs per SM
 // with large NB.  Measured on the rings: CTAs of 64 and 96 threads 2 to 6 % slower, of 256 threads 3 % (NB = 6) to 20 %
-// (NB = 10, 14), half as many lines 23 % slower for NB = 3.
+// (NB = 10, 14), half as many lines 23 % slower for NB = 3.  Lines of one or two M-point steps come from boxes of a few
+// thousand lines: small CTAs spread their arithmetic over the chip (32^3 cells in FP64, 32 lines and 128 threads per CTA:
+// 92 us, these: 72 us; in double-float, one component, 53 and 42 us).
 template <int M, int NB>
 struct LineTile {
-  static constexpr int NT = 128;
-  static constexpr int TL = NB <= 2 ? 32 : (NB <= 5 ? 16 : 8);
+  static constexpr int NT = NB <= 2 ? 64 : 128;
+  static constexpr int TL = NB == 2 ? 8 : (NB <= 5 ? 16 : 8);
   // CTAs per SM that the registers are limited for: 80 registers up to NB = 6 (the M-point step alone holds 64),
   // more for the NB-point step of wide boxes, where spills cost more than the occupancy gains
-  static constexpr int MB = NB <= 6 ? 6 : (NB == 7 ? 5 : (NB <= 10 ? 4 : (NB < 16 ? 3 : 2)));
+  static constexpr int MB = NB <= 2 ? 12 : NB <= 6 ? 6 : (NB == 7 ? 5 : (NB <= 10 ? 4 : (NB < 16 ? 3 : 2)));
 };
 
 // 4- or 8-byte asynchronous copies to shared memory, and the wait for the thread's own.
