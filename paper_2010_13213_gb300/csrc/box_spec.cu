@@ -200,7 +200,7 @@ static int line_rows(const BoxSpec *S, int B, typename Ar<R>::T **dst, cudaStrea
 // K1 = 2 (k3 N2 + k2) + h holds K = 2 K' + h with K' = k3 mod NO, K' = k2 + N2 K2 mod M N2; a real field keeps the
 // slots that are not above their mirror, in order.
 static int line_freqs(BoxSpec *S, int B, cudaStream_t st) {
-  const int nb = S->nb[0], M = B == 8 && nb % 2 ? 8 : 16, NB = nb * B / M;
+  const int nb = S->nb[0], M = line_M(B, nb), NB = line_NB(B, nb);
   const int N2 = NB & -NB, NO = NB / N2, Q2 = M * N2, n = M * NB;
   auto freq = [&](int k1, int k2big) {  // by search: tables of at most 512 entries
     const int q = k1 / 2, k3 = q / N2, kk = q % N2 + N2 * k2big;
@@ -286,7 +286,7 @@ static int gen_spectrum(lgf_table *t, BoxSpec *S, cudaStream_t st) {
     if (cudaMalloc(&wP[a], sizeof(cx<double>) * g.P[a])) return fail(LGF_E_OOM, "tables");
     cudaMemcpyAsync(wP[a], w.data(), sizeof(cx<double>) * g.P[a], cudaMemcpyHostToDevice, st);
     for (int i = 0; i < g.P[a] && i < 32; ++i) S->bw32[a][i] = cx<float>{(float)c[i], -(float)s[i]};
-    const int P = 2 * g.nb[a] * B / (B == 8 && g.nb[a] % 2 ? 8 : 16);  // 2 NB of the line transforms
+    const int P = 2 * line_NB(B, g.nb[a]);  // 2 NB of the line transforms
     line_tables<double>(P, S->lt64[a]);
     line_tables<float>(P, S->lt32[a]);
     line_tables<df>(P, S->ltdf[a]);

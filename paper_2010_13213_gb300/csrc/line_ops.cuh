@@ -22,10 +22,6 @@ struct LinePass {
   cudaStream_t st = nullptr;
 };
 
-// Points of the second step and block count of a line of nb blocks of B cells.
-inline int line_M(int B, int nb) { return B == 8 && nb % 2 ? 8 : 16; }
-inline int line_NB(int B, int nb) { return nb * B / line_M(B, nb); }
-
 template <class K>
 inline void line_smem_limit(K kern, size_t sm, bool &done) {
   if (done) return;
@@ -97,7 +93,9 @@ bool line_range(int nb, LineKind kind, const LinePass<R> &p);
   template <>                                                                       \
   bool line_range<R, 16, 12, 16, 1>(int, LineKind, const LinePass<R> &);            \
   template <>                                                                       \
-  bool line_range<R, 8, 1, 15, 2>(int, LineKind, const LinePass<R> &);
+  bool line_range<R, 8, 1, 15, 2>(int, LineKind, const LinePass<R> &);              \
+  template <>                                                                       \
+  bool line_range<R, 8, 2, 2, 1>(int, LineKind, const LinePass<R> &);
 LINE_RANGE_DECLARE(double)
 LINE_RANGE_DECLARE(float)
 LINE_RANGE_DECLARE(df)
@@ -105,6 +103,7 @@ LINE_RANGE_DECLARE(df)
 template <class R>
 inline bool line_pass(int B, int nb, LineKind kind, const LinePass<R> &p) {
   const int NB = line_NB(B, nb);
+  if (line_M(B, nb) == 8 && NB == 2) return line_range<R, 8, 2, 2, 1>(NB, kind, p);
   if (line_M(B, nb) == 8) return line_range<R, 8, 1, 15, 2>(NB, kind, p);
   if (NB <= 6) return line_range<R, 16, 1, 6, 1>(NB, kind, p);
   if (NB <= 11) return line_range<R, 16, 7, 11, 1>(NB, kind, p);
