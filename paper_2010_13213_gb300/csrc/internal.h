@@ -105,9 +105,10 @@ struct TcMat {
 };
 
 // Points M of the second step and count NB of the first step of a box line of nb blocks of B cells, M NB cells.  Two
-// 8^3 blocks take 8-point steps as odd counts must: one 16-point transform per line is one long chain
-// (16^3 cells: FP64 64 us with 16-point steps, 42 with 8; double-float 40 and 29).
-inline int line_M(int B, int nb) { return B == 8 && (nb % 2 || nb == 2) ? 8 : 16; }
+// and four 8^3 blocks take 8-point steps as odd counts must: 16-point transforms of short lines are long chains on few
+// threads (16^3 cells: FP64 64 us with 16-point steps, 42 with 8, double-float 40 and 29; 32^3 cells of 8^3 blocks,
+// three components: 108 and 81, 51 and 42; boxes with one axis of four blocks and others of six or seven 2 to 14 %).
+inline int line_M(int B, int nb) { return B == 8 && (nb % 2 || nb <= 4) ? 8 : 16; }
 inline int line_NB(int B, int nb) { return nb * B / line_M(B, nb); }
 
 struct BoxSpec {

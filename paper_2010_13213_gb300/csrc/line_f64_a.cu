@@ -3,5 +3,5 @@
 
 namespace lgf {
 LINE_RANGE_DEFINE(double, 16, 1, 6, 1)
-LINE_RANGE_DEFINE(double, 8, 2, 2, 1)
+LINE_RANGE_DEFINE(double, 8, 2, 4, 2)
 }  // namespace lgf

@@ -95,7 +95,7 @@ bool line_range(int nb, LineKind kind, const LinePass<R> &p);
   template <>                                                                       \
   bool line_range<R, 8, 1, 15, 2>(int, LineKind, const LinePass<R> &);              \
   template <>                                                                       \
-  bool line_range<R, 8, 2, 2, 1>(int, LineKind, const LinePass<R> &);
+  bool line_range<R, 8, 2, 4, 2>(int, LineKind, const LinePass<R> &);
 LINE_RANGE_DECLARE(double)
 LINE_RANGE_DECLARE(float)
 LINE_RANGE_DECLARE(df)
@@ -103,7 +103,7 @@ LINE_RANGE_DECLARE(df)
 template <class R>
 inline bool line_pass(int B, int nb, LineKind kind, const LinePass<R> &p) {
   const int NB = line_NB(B, nb);
-  if (line_M(B, nb) == 8 && NB == 2) return line_range<R, 8, 2, 2, 1>(NB, kind, p);
+  if (line_M(B, nb) == 8 && NB % 2 == 0) return line_range<R, 8, 2, 4, 2>(NB, kind, p);
   if (line_M(B, nb) == 8) return line_range<R, 8, 1, 15, 2>(NB, kind, p);
   if (NB <= 6) return line_range<R, 16, 1, 6, 1>(NB, kind, p);
   if (NB <= 11) return line_range<R, 16, 7, 11, 1>(NB, kind, p);
