@@ -64,7 +64,7 @@ struct RefreshPlan {
 static std::mutex g_rp_mu;
 static std::list<std::pair<std::string, std::shared_ptr<RefreshPlan>>> g_rp;  // most recent first
 
-static int refresh_plan(const lgf_mesh *m, std::shared_ptr<RefreshPlan> &out) {
+static int refresh_plan(const lgf_mesh *m, std::shared_ptr<RefreshPlan> &out, cudaStream_t st) {
   const int n = m->nblocks[0];
   int dev = 0;
   cudaGetDevice(&dev);
@@ -102,8 +102,13 @@ static int refresh_plan(const lgf_mesh *m, std::shared_ptr<RefreshPlan> &out) {
     cudaGetLastError();
     return set_error(LGF_E_OOM, "velocity refresh neighbour table");
   }
-  if (cudaMemcpy(P->d_nbr, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+  // on the device before any stream can find the plan: a copy from pageable memory on the legacy stream may return before
+  // the transfer has ended, and the caller's streams do not wait for that stream
+  if (cudaMemcpyAsync(P->d_nbr, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess) {
+    cudaGetLastError();
     return set_error(LGF_E_CUDA, "velocity refresh neighbour table upload");
+  }
   g_rp.emplace_front(key, P);
   while (g_rp.size() > 1024) g_rp.pop_back();  // cudaFree inside orders against in-flight work
   out = P;
@@ -134,7 +139,7 @@ extern "C" int lgf_velocity_refresh(lgf_table *t, const lgf_mesh *m, const void 
   const int shift = B == 8 ? 3 : 4;
   const int64_t B3 = (int64_t)B * B * B;
   std::shared_ptr<RefreshPlan> P;
-  if ((rc = refresh_plan(m, P))) return rc;
+  if ((rc = refresh_plan(m, P, st))) return rc;
   const int next = P->next;
   lgf_mesh me = *m;
   const int32_t nb_ext[1] = {next};
