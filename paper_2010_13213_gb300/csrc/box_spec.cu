@@ -254,6 +254,19 @@ static int block_twiddles(BoxSpec *S, const BoxGeom &g, int B, cudaStream_t st) 
   return set_error(LGF_E_OOM, "box spectrum: twiddles");
 }
 
+// The block-index paths' tables, from the folded spectrum.
+static int gen_blocks(BoxSpec *S, int B, cudaStream_t st) {
+  const BoxGeom g = spec_geom(S);
+  const int64_t n = (int64_t)g.P[0] * g.P[1] * g.P[2] * B * B * B;
+  if (cudaMalloc(&S->g32, sizeof(float) * n) != cudaSuccess || cudaMalloc(&S->gdf, sizeof(df) * n) != cudaSuccess) {
+    cudaGetLastError();
+    return set_error(LGF_E_OOM, "block-order spectrum");
+  }
+  S->bytes += (size_t)n * 12;
+  k_spec_unfold<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(S->gf64, B, g, n, S->g32, S->gdf);
+  return tc_matrices(S, g, st);  // synchronises
+}
+
 template <int B>
 static int gen_spectrum(lgf_table *t, BoxSpec *S, cudaStream_t st) {
   constexpr int B3 = B * B * B;
@@ -316,26 +329,10 @@ static int gen_spectrum(lgf_table *t, BoxSpec *S, cudaStream_t st) {
   release();
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess)
     return set_error(LGF_E_CUDA, "box spectrum kernels failed: %s", cudaGetErrorString(e));
-  return LGF_OK;
+  return gen_blocks(S, B, st);
 }
 
-// The block-index paths' tables, from the folded spectrum.
-static int gen_blocks(BoxSpec *S, int B, cudaStream_t st) {
-  const BoxGeom g = spec_geom(S);
-  const int64_t n = (int64_t)g.P[0] * g.P[1] * g.P[2] * B * B * B;
-  if ((!S->g32 && cudaMalloc(&S->g32, sizeof(float) * n) != cudaSuccess) ||
-      (!S->gdf && cudaMalloc(&S->gdf, sizeof(df) * n) != cudaSuccess)) {
-    cudaGetLastError();
-    return set_error(LGF_E_OOM, "block-order spectrum");
-  }
-  S->bytes += (size_t)n * 12;
-  k_spec_unfold<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(S->gf64, B, g, n, S->g32, S->gdf);
-  const int rc = tc_matrices(S, g, st);  // synchronises
-  if (!rc) S->blocks_ready = true;
-  return rc;
-}
-
-int box_spectrum(lgf_table *t, const int nb[3], bool blocks, BoxSpec **out, cudaStream_t st) {
+int box_spectrum(lgf_table *t, const int nb[3], BoxSpec **out, cudaStream_t st) {
   for (int a = 0; a < 3; ++a) {
     if (nb[a] < 1 || nb[a] > BOX_NB_MAX)
       return set_error(LGF_E_UNSUPPORTED, "box mode supports 1..%d blocks per axis (got %d)", BOX_NB_MAX, nb[a]);
@@ -356,8 +353,6 @@ int box_spectrum(lgf_table *t, const int nb[3], bool blocks, BoxSpec **out, cuda
     }
     t->box[key] = S;
   }
-  if (blocks && !S->blocks_ready)
-    if (const int rc = gen_blocks(S, t->B, st)) return rc;
   *out = S;
   return LGF_OK;
 }

@@ -127,12 +127,9 @@ struct BoxSpec {
   Ar<df>::T *ltldf = nullptr;
   int ltl_off[3] = {0, 0, 0};
   int32_t *fx = nullptr;  // x frequency per row element: complex fields (2 nb_x B of them), then real fields
-  // the tensor-core DFT-GEMM (box_tc.cuh), the FP32 passes of box_pass.cuh and k_box_mid, built on the first solve that
-  // uses one of them: the spectrum in
-  // block order [P^3 blocks][B^3], the coefficient digits, and the four-step twiddles W_L^n, n < L = lcm(Pcx, Pcy,
-  // Pcz) (Pc = P B cells per axis; the twiddle of a cell m and block frequency K1 is
-  // W_L^{(sum_a m_a K1_a L / Pc_a) mod L})
-  bool blocks_ready = false;
+  // the tensor-core DFT-GEMM (box_tc.cuh), the FP32 passes of box_pass.cuh and k_box_mid: the spectrum in block order
+  // [P^3 blocks][B^3], the coefficient digits, and the four-step twiddles W_L^n, n < L = lcm(Pcx, Pcy, Pcz) (Pc = P B
+  // cells per axis; the twiddle of a cell m and block frequency K1 is W_L^{(sum_a m_a K1_a L / Pc_a) mod L})
   cx<float> bw32[3][32];    // W_P^n per axis, n < P (host copies for kernel parameters)
   float *g32 = nullptr;
   df *gdf = nullptr;
@@ -185,15 +182,13 @@ struct Workspace {
 namespace lgf {
 // FP32 arithmetic on FP64 fields runs the block-index passes (box_pass.cuh says why).
 inline bool box_blocks(const lgf_solve_opts &o, int dtype) { return o.precision == LGF_PREC_FP32 && dtype == LGF_F64; }
-// The spectrum and tables of a box shape, built on first use; `blocks`: with those of the block-index paths.
-int box_spectrum(lgf_table *t, const int nb[3], bool blocks, BoxSpec **out, cudaStream_t st);
-// Bytes of the two scratch arrays of BoxOps::convolve for `nf` complex fields of `csize` bytes a value on `cells`
-// box cells: the line passes hold the x-transformed and the x- and y-transformed fields (2 and 4 values a cell),
-// the block-index passes the whole padded box twice.
-inline void box_scratch(int64_t nf, int64_t cells, size_t csize, bool blocks, size_t bytes[2]) {
-  bytes[0] = (size_t)nf * cells * csize * (blocks ? 8 : 2);
-  bytes[1] = (size_t)nf * cells * csize * (blocks ? 8 : 4);
-}
+// The spectrum and tables of a box shape, built on first use: those of every evaluation, so that a mesh solved once may be
+// captured, or solved on another stream, with other options.
+int box_spectrum(lgf_table *t, const int nb[3], BoxSpec **out, cudaStream_t st);
+// Bytes of each of the two scratch arrays of BoxOps::convolve for `nf` complex fields of `csize` bytes a value on `cells`
+// box cells, whichever evaluation runs: the block-index passes hold the whole padded box (8 values a cell), the line
+// passes the x-transformed and the x- and y-transformed fields (2 and 4).
+inline size_t box_scratch(int64_t nf, int64_t cells, size_t csize) { return (size_t)nf * cells * csize * 8; }
 // Synchronous read of the table's device status word; LGF_E_TIMEOUT (and the word cleared) when a
 // bounded device-side wait gave up since the last read.
 int take_device_status(lgf_table *t);

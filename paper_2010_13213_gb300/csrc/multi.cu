@@ -197,10 +197,9 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
                        Gh ? "box support for it" : "pair spectra of this precision");
   Workspace *ws = workspace_for(t, st);
   const size_t field = sizeof(R) * (size_t)ncomp * maxBL * B3;
-  size_t ybytes[2];
-  box_scratch(std::min(ncomp, BOX_MAXF), maxbox, sizeof(cx<R>), o.dft_slices > 0 || box_blocks(o, dtype), ybytes);
-  if ((rc = ws->buf[0].reserve(std::max(ybytes[0], sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSA, 1) * W))) ||
-      (rc = ws->buf[1].reserve(std::max(ybytes[1], sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxT, 1) * W))) ||
+  const size_t ybytes = box_scratch(std::min(ncomp, BOX_MAXF), maxbox, sizeof(cx<R>));
+  if ((rc = ws->buf[0].reserve(std::max(ybytes, sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSA, 1) * W))) ||
+      (rc = ws->buf[1].reserve(std::max(ybytes, sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxT, 1) * W))) ||
       (rc = ws->buf[3].reserve(sizeof(cx<R>) * (size_t)ncomp * std::max<int64_t>(maxSB, 1) * W)) ||
       (rc = ws->buf[4].reserve(sizeof(R) * (size_t)Foff[K])) || (rc = ws->buf[5].reserve(field)) ||
       (rc = ws->buf[6].reserve(field)) || (rc = ws->buf[7].reserve(sizeof(R) * (size_t)Foff[K])) ||
@@ -272,7 +271,7 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
     }
     if (use_box[k]) {
       BoxSpec *S = nullptr;
-      if ((rc = box_spectrum(t, L.box_nb, o.dft_slices > 0 || box_blocks(o, dtype), &S, st))) return rc;
+      if ((rc = box_spectrum(t, L.box_nb, &S, st))) return rc;
       const int32_t *gA = L.d_box, *gB = gA + L.nbox, *sPsi = gB + L.nbox, *sPhi = sPsi + L.nbox;
       const double hk = m->h0 / (double)(1 << k);
       const double scale = hk * hk;

@@ -257,13 +257,12 @@ static int solve_single_box(lgf_table *t, const lgf_mesh *m, const SinglePlan *P
   const int B = m->block, n = m->nblocks[0];
   const int64_t B3 = (int64_t)B * B * B;
   BoxSpec *S = nullptr;
-  int rc = box_spectrum(t, P->nb, o.dft_slices > 0 || box_blocks(o, dtype), &S, st);
+  int rc = box_spectrum(t, P->nb, &S, st);
   if (rc) return rc;
   Workspace *ws = workspace_for(t, st);
   const int nf = (ncomp + 1) / 2;
-  size_t ybytes[2];
-  box_scratch(std::min(nf, BOX_MAXF), P->nbox * B3, sizeof(cx<R>), o.dft_slices > 0 || box_blocks(o, dtype), ybytes);
-  if ((rc = ws->buf[0].reserve(ybytes[0])) || (rc = ws->buf[1].reserve(ybytes[1]))) return rc;
+  const size_t ybytes = box_scratch(std::min(nf, BOX_MAXF), P->nbox * B3, sizeof(cx<R>));
+  if ((rc = ws->buf[0].reserve(ybytes)) || (rc = ws->buf[1].reserve(ybytes))) return rc;
   const int32_t *gmap = P->d_idx + P->nsrc + P->ntgt, *smap = gmap + P->nbox;
   PhaseTimer tm;
   tm.start(o.timing != 0, st);
