@@ -83,16 +83,13 @@ static void tc_pass_launch(const cx<R> *in, cx<R> *out, int64_t fstride, const B
                            const TcMat &M, int gather, int final, int nfield, int lines, const FwdSpecs &sp,
                            const InvOuts<R> &outs, double sc, int *status, cudaStream_t st) {
   static int nsm = 0;
-  static bool attr = false;
+  static PerDevice limit;
   if (!nsm) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   }
-  if (!attr) {
-    cudaFuncSetAttribute(k_bdft_tc<R, B, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr = true;
-  }
+  smem_limit(limit, k_bdft_tc<R, B, SL>, 227 * 1024);
   const TcSmem pl = tc_smem_plan(SL, M.Kp, M.Np);
   uint32_t cols = 32;
   while (cols < (uint32_t)(SL * M.Np)) cols <<= 1;
@@ -205,11 +202,8 @@ static int box_group_blocks(const BoxSpec *S, const std::vector<int> &fields, in
   const int pxu = box_pxmax(g);  // lines of the y and z passes run over the widest K1x range
   const int64_t nmid = (int64_t)pxu * P[1] * P[2];
   const size_t sm = sizeof(cx<R>) * (size_t)B * B * (B + 1);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_box_mid<R, B, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static PerDevice limit;
+  smem_limit(limit, k_box_mid<R, B, true>, sm);
   const int n = (int)fields.size();
   FwdSpecs sp{};
   InvOuts<R> outs{};

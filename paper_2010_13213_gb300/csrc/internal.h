@@ -13,8 +13,19 @@
 #include "../../include/lgf.h"
 #include "arith.cuh"
 #include "common.cuh"
+#include "per_device.h"
 
 namespace lgf {
+
+// The dynamic shared memory limit of a kernel on the current device, set on the first call there (`done`: one per kernel).
+template <class K>
+inline void smem_limit(PerDevice &done, K kern, size_t bytes) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  done.run(dev, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  });
+}
 
 int set_error(int code, const char *fmt, ...);
 int check_slices(const lgf_solve_opts &o);

@@ -22,43 +22,36 @@ struct LinePass {
   cudaStream_t st = nullptr;
 };
 
-template <class K>
-inline void line_smem_limit(K kern, size_t sm, bool &done) {
-  if (done) return;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  done = true;
-}
-
 template <class R, int M, int NB>
 void line_launch(LineKind kind, const LinePass<R> &p) {
   constexpr int TL = LineTile<M, NB>::TL, NT = LineTile<M, NB>::NT;
   constexpr size_t smx = line_smem<R, M, NB, true>(), smy = line_smem<R, M, NB, false>(),
                    smm = line_smem_mid<R, M, NB>();
-  static bool done[5] = {};
+  static PerDevice done[5];
   const unsigned tiles_yz = (unsigned)((p.g.n[1] * p.g.n[2] + TL - 1) / TL), tiles_w = (unsigned)((p.wmax + TL - 1) / TL);
   const unsigned nz = (unsigned)p.g.n[2], nf = (unsigned)p.nfields;
   switch (kind) {
     case LINE_FWD_X:
-      line_smem_limit(k_line_fwd<R, M, NB, true>, smx, done[kind]);
+      smem_limit(done[kind], k_line_fwd<R, M, NB, true>, smx);
       k_line_fwd<R, M, NB, true><<<dim3(tiles_yz, 1, nf), NT, smx, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.sp);
       break;
     case LINE_FWD_Y:
-      line_smem_limit(k_line_fwd<R, M, NB, false>, smy, done[kind]);
+      smem_limit(done[kind], k_line_fwd<R, M, NB, false>, smy);
       k_line_fwd<R, M, NB, false><<<dim3(tiles_w, nz, nf), NT, smy, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.sp);
       break;
     case LINE_MID: {
       const unsigned tiles = (unsigned)(((int64_t)p.g.P[1] * p.g.M[1] * p.wmax + TL - 1) / TL);
-      line_smem_limit(k_line_mid<R, M, NB>, smm, done[kind]);
+      smem_limit(done[kind], k_line_mid<R, M, NB>, smm);
       k_line_mid<R, M, NB><<<dim3(tiles, 1, nf), NT, smm, p.st>>>(p.out, p.Gf, p.g, *p.tw, p.twl);
       break;
     }
     case LINE_INV_Y:
-      line_smem_limit(k_line_inv<R, M, NB, false>, smy, done[kind]);
+      smem_limit(done[kind], k_line_inv<R, M, NB, false>, smy);
       k_line_inv<R, M, NB, false><<<dim3(tiles_w, nz, nf), NT, smy, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
                                                                            1.0);
       break;
     case LINE_INV_X:
-      line_smem_limit(k_line_inv<R, M, NB, true>, smx, done[kind]);
+      smem_limit(done[kind], k_line_inv<R, M, NB, true>, smx);
       k_line_inv<R, M, NB, true><<<dim3(tiles_yz, 1, nf), NT, smx, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
                                                                           p.scale);
       break;

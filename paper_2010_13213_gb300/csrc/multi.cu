@@ -33,13 +33,11 @@ double box_cost(int B, const int nb[3]);
 double pair_cost(int B, double nsrc, double ntgt);
 
 // Dynamic shared memory of k_correct with the correction (the staged c cube; with the static coarse cube
-// above the default 48 KB for 8-byte arithmetics, so the limit is raised once per arithmetic).
+// above the default 48 KB for 8-byte arithmetics, so the limit is raised once per arithmetic and device).
 template <class R>
 static size_t correct_smem(int B) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_correct<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)halo_smem<R>(16));
-  });
+  static PerDevice limit;
+  smem_limit(limit, k_correct<R>, halo_smem<R>(16));
   return halo_smem<R>(B);
 }
 
@@ -524,19 +522,12 @@ static int heat_weights(double alpha, HeatW *w) {
 template <class R, int BB>
 static int heat_line_launch(const LevelDev &Ld, const int4 *BL, const int32_t *HB, int nHB, int ncomp, int ax,
                             const R *in, R *out, int64_t cs, const HeatW &w, cudaStream_t st) {
-  static bool attr = false;
+  static PerDevice limit;
   if constexpr (std::is_same<R, df>::value) {
-    if (!attr) {
-      cudaFuncSetAttribute(k_heat_pair<BB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)heat_pair_smem<BB>(BB));
-      attr = true;
-    }
+    smem_limit(limit, k_heat_pair<BB>, heat_pair_smem<BB>(BB));
     k_heat_pair<BB><<<dim3(nHB, ncomp), BB * BB / 2, heat_pair_smem<BB>(w.r), st>>>(Ld, BL, HB, ax, in, out, cs, w);
   } else {
-    if (!attr) {
-      cudaFuncSetAttribute(k_heat_line<R, BB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)heat_line_smem<R, BB>(BB));
-      attr = true;
-    }
+    smem_limit(limit, k_heat_line<R, BB>, heat_line_smem<R, BB>(BB));
     k_heat_line<R, BB><<<dim3(nHB, ncomp), BB * BB, heat_line_smem<R, BB>(w.r), st>>>(Ld, BL, HB, ax, in, out, cs, w);
   }
   cudaError_t e = cudaGetLastError();

@@ -10,11 +10,8 @@ static int fwd_b(const void *f, int dtype, int64_t cs, const int32_t *src_idx, i
                  void *spec, const uint8_t *cellmask, int bits, cudaStream_t st) {
   if (nsrc == 0) return LGF_OK;
   const size_t sm = pair_fft_smem<R, B>();
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_block_fwd<R, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static PerDevice limit;
+  smem_limit(limit, k_block_fwd<R, B>, sm);
   k_block_fwd<R, B><<<dim3(nsrc, ncomp), 256, sm, st>>>(f, dtype, cs, src_idx, nsrc, (cx<R> *)spec,
                                                         cellmask, bits, make_tw64<R>());
   cudaError_t e = cudaGetLastError();
@@ -27,11 +24,8 @@ static int inv_b(const void *spec, int64_t spec_cs, const int32_t *rows, const i
                  const uint8_t *cellmask, int bits, double scale, cudaStream_t st) {
   if (n == 0) return LGF_OK;
   const size_t sm = pair_fft_smem<R, B>();
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_block_inv<R, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static PerDevice limit;
+  smem_limit(limit, k_block_inv<R, B>, sm);
   k_block_inv<R, B><<<dim3(n, ncomp), 256, sm, st>>>((const cx<R> *)spec, spec_cs, rows, aux, out, dtype, out_cs,
                                                      out_off, (const R *)addend, add_cs, cellmask, bits, scale,
                                                      make_tw64<R>());
