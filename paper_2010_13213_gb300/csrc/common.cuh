@@ -40,15 +40,16 @@ LGF_D df df_make(double v) {
   float l = __double2float_rn(v - (double)h);
   return {h, l};
 }
-// hi + lo in double: within 2^-100 <= |hi| < 2^127 the low part, rounded to hi's 2^-29 ulp, is added to hi's bit
-// pattern (no FP64 instruction, see df_make); |lo| <= ulp(hi) (a renormalised value).
+// hi + lo in double, correctly rounded: within 2^-100 <= |hi| < 2^127 the low part, rounded to an ulp of the result, is
+// added to hi's bit pattern (no FP64 instruction, see df_make); |lo| <= ulp(hi) (a renormalised value).
 LGF_D double df_to_double(df a) {
   const unsigned hb = __float_as_uint(a.hi), e = (hb >> 23) & 0xffu;
   const float rel = __fmul_rn(a.lo, __uint_as_float((254u - e) << 23));  // lo / 2^exponent(hi)
   if (e - 27u < 227u && fabsf(rel) <= 1.1920928955078125e-7f) {          // 2^-23
-    int q = __float2int_rn(__fmul_rn(rel, 4503599627370496.0f));         // 2^52
-    q = (hb >> 31) ? -q : q;                                             // towards (+) or away from hi's magnitude
-    if (q < 0 && !(hb & 0x7fffffu)) q *= 2;                              // below a power of two the ulp halves
+    // ulps of the result: 2^-52 of hi's power of two, half of that below it
+    const bool below = !(hb & 0x7fffffu) && ((hb ^ __float_as_uint(rel)) >> 31);
+    int q = __float2int_rn(__fmul_rn(rel, below ? 9007199254740992.0f : 4503599627370496.0f));  // 2^53, 2^52
+    q = (hb >> 31) ? -q : q;  // towards (+) or away from hi's magnitude
     const unsigned lw = hb << 29, hw = (((hb & 0x7fffffffu) >> 3) + 0x38000000u) | (hb & 0x80000000u);
     const long long bits = (long long)(((unsigned long long)hw << 32) | lw) + (long long)q;
     return __longlong_as_double(bits);
