@@ -398,9 +398,10 @@ int BoxOps<R>::convolve(int B, const BoxSpec *S, int nf, const int *nin, const I
       for (int f : grp) nc += std::find(cplx.begin(), cplx.end(), f) != cplx.end();
       int rc = LGF_OK;
       if (slices == 0 && !blocks) {
-        // the double-float Ghat carries the 1 / (8 cells) of the inverse transform
-        rc = box_group_lines<R>(B, S, grp, nc, nin, in, ore, oim, std::is_same<R, df>::value ? scale : scale / cells8, Y0,
-                                Y1, st, mark, mark_ctx);
+        // the double-float Ghat carries the rest of the 1 / (8 cells) of the inverse transform
+        rc = box_group_lines<R>(B, S, grp, nc, nin, in, ore, oim,
+                                scale / (std::is_same<R, df>::value ? box_pow2((int64_t)cells8) : cells8), Y0, Y1, st, mark,
+                                mark_ctx);
       } else if constexpr (!std::is_same<R, double>::value) {
         rc = B == 8 ? box_group_blocks<R, 8>(S, grp, nc, nin, in, ore, oim, scale / cells8, Y0, Y1, st, mark, mark_ctx,
                                              slices, status)

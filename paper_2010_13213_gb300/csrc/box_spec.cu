@@ -18,7 +18,7 @@ namespace lgf {
 
 // Ghat on the folded lattice [f_z][f_y][f_x], 0 <= f_a <= Pc_a / 2, from block order (k_box_mid: [K1 block][x][z][y],
 // f = K1 + P K2 per axis); n = values.
-__global__ void k_spec_fold(const double *__restrict__ g, int B, BoxGeom geo, int64_t n, double inv8, double *__restrict__ g64,
+__global__ void k_spec_fold(const double *__restrict__ g, int B, BoxGeom geo, int64_t n, double mant8, double *__restrict__ g64,
                             float *__restrict__ g32, df *__restrict__ gdf) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -28,9 +28,10 @@ __global__ void k_spec_fold(const double *__restrict__ g, int B, BoxGeom geo, in
   const double v = g[((kb * B + fx / geo.P[0]) * B + fz / geo.P[2]) * B + fy / geo.P[1]];
   g64[i] = v;
   g32[i] = (float)v;
-  // with the 1 / (8 cells) of the inverse transform: the last pass then scales by h^2, which rounds nothing for a
-  // power of two (error of the two rings 5.8e-15 -> 5.0e-15)
-  gdf[i] = df_make(v * inv8);
+  // with the 1 / (8 cells) of the inverse transform up to a power of two: the last pass then scales by h^2 and that
+  // power, which rounds nothing for an h that is one (error of the two rings 5.8e-15 -> 5.0e-15).  The power stays out, as
+  // it would take low parts of small fields below the floats' range.
+  gdf[i] = df_make(v * mant8);
 }
 
 // Block order from the folded spectrum (k_box_mid of the block-index paths); n = P^3 B^3 values.
@@ -323,7 +324,7 @@ static int gen_spectrum(lgf_table *t, BoxSpec *S, cudaStream_t st) {
   cudaFuncSetAttribute(k_box_mid<double, B, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_box_mid<double, B, false><<<dim3((unsigned)nblk, 1), mid_threads<double, B>(), sm, st>>>(
       Y0, 0, nullptr, g, S->twl64, S->twL, make_int3(S->twf[0], S->twf[1], S->twf[2]), make_tw64<double>(), block_order);
-  k_spec_fold<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(block_order, B, g, nf, 1.0 / (double)n, S->gf64, S->gf32,
+  k_spec_fold<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(block_order, B, g, nf, box_pow2(n) / (double)n, S->gf64, S->gf32,
                                                           S->gfdf);
   const cudaError_t e = cudaStreamSynchronize(st);
   release();

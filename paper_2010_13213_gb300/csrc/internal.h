@@ -196,6 +196,9 @@ inline bool box_blocks(const lgf_solve_opts &o, int dtype) { return o.precision 
 // The spectrum and tables of a box shape, built on first use: those of every evaluation, so that a mesh solved once may be
 // captured, or solved on another stream, with other options.
 int box_spectrum(lgf_table *t, const int nb[3], BoxSpec **out, cudaStream_t st);
+// The largest power of two that is not above n: of the 1 / (8 cells) of a box, gfdf carries box_pow2 / (8 cells), and the
+// last pass 1 / box_pow2.
+inline double box_pow2(int64_t n) { return ldexp(1.0, ilogb((double)n)); }
 // Bytes of each of the two scratch arrays of BoxOps::convolve for `nf` complex fields of `csize` bytes a value on `cells`
 // box cells, whichever evaluation runs: the block-index passes hold the whole padded box (8 values a cell), the line
 // passes the x-transformed and the x- and y-transformed fields (2 and 4).
