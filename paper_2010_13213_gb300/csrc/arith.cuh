@@ -11,7 +11,8 @@
 // the FP32 pipe instead of 80 %.
 //
 // Double-float sums and real products are left unnormalised (lazy: TwoSum of the high parts, plain sums of the low
-// parts); callers renormalise (norm) before a value enters a complex product, which renormalises its result.  Products by i swap the halves of a pair, with the sign folded into an exact multiply by
+// parts); callers renormalise (norm) before a value enters a complex product, which renormalises its result.  ArFine
+// renormalises every sum.  Products by i swap the halves of a pair, with the sign folded into an exact multiply by
 // (+1, -1) inside the following sum.
 #pragma once
 #include "common.cuh"
@@ -62,6 +63,7 @@ struct Ar;
 // ------------------------------------------------------------------ double
 template <>
 struct Ar<double> {
+  typedef double Real;
   struct V {
     double re, im;
   };
@@ -98,6 +100,7 @@ struct Ar<double> {
 // ------------------------------------------------------------------ float
 template <>
 struct Ar<float> {
+  typedef float Real;
   struct V {
     f2 v;
   };
@@ -138,6 +141,7 @@ struct Ar<float> {
 // ------------------------------------------------------------------ double-float
 template <>
 struct Ar<df> {
+  typedef df Real;
   struct V {
     f2 h, l;
   };
@@ -221,6 +225,24 @@ struct Ar<df> {
   static LGF_D V scale_conj(V a, df g) { return mulr(a, f2_pack(g.hi, -g.hi), f2_pack(g.lo, -g.lo)); }
 };
 
+// The same arithmetic with every double-float sum and real product renormalised, 11 packed instructions a sum instead of
+// 8: a sum of lazy sums rounds in proportion to low parts of several ulps.
+template <class R>
+struct ArFine : Ar<R> {};
+template <>
+struct ArFine<df> : Ar<df> {
+  typedef Ar<df> L;
+  static LGF_D V add(V a, V b) { return norm(L::add(a, b)); }
+  static LGF_D V sub(V a, V b) { return norm(L::sub(a, b)); }
+  static LGF_D V add_mi(V a, V b) { return norm(L::add_mi(a, b)); }
+  static LGF_D V add_pi(V a, V b) { return norm(L::add_pi(a, b)); }
+  static LGF_D V add_mh(V a, V b) { return norm(L::add_mh(a, b)); }
+  static LGF_D V fma_re(V acc, V a, T w) { return norm(L::fma_re(acc, a, w)); }
+  static LGF_D V fma_im(V acc, V s, T w) { return norm(L::fma_im(acc, s, w)); }
+  static LGF_D V mul_im(V s, T w) { return norm(L::mul_im(s, w)); }
+  static LGF_D V mul_w8(V v, T w) { return norm(mulr(add_mi(v, v), w.reh, w.rel)); }
+};
+
 // Host-side construction of a twiddle (re, im) from FP64 (T as above).
 inline void make_T(double re, double im, Ar<double>::T &t) { t = make_double2(re, im); }
 inline f2 host_pack(float a, float b) {
@@ -245,7 +267,7 @@ inline void make_T(double re, double im, Ar<df>::T &t) {
 }
 
 // ------------------------------------------------------------------ small DFTs in registers
-// Forward DFTs (e^{-2 pi i jk / N}), unnormalised, natural order in and out.
+// Forward DFTs (e^{-2 pi i jk / N}), unnormalised, natural order in and out; A is Ar<R> or ArFine<R>.
 
 // Twiddles of one launch, in the parameter bank: W_P^n, n < P = 2 NB, and the constants of the 16-point FFT.
 #define LINE_P_MAX 32
@@ -257,9 +279,8 @@ struct LineTw {
 };
 
 // 4 points; the third and fourth input may come without their factor -i (M2, M3), folded into the sums.
-template <class R, bool M2 = false, bool M3 = false>
-LGF_D void dft4(typename Ar<R>::V &a, typename Ar<R>::V &b, typename Ar<R>::V &c, typename Ar<R>::V &d) {
-  typedef Ar<R> A;
+template <class A, bool M2 = false, bool M3 = false>
+LGF_D void dft4(typename A::V &a, typename A::V &b, typename A::V &c, typename A::V &d) {
   const typename A::V s02 = M2 ? A::add_mi(a, c) : A::add(a, c), d02 = M2 ? A::add_pi(a, c) : A::sub(a, c);
   const typename A::V s13 = M3 ? A::add_mi(b, d) : A::add(b, d), d13 = M3 ? A::add_pi(b, d) : A::sub(b, d);
   a = A::add(s02, s13);
@@ -275,11 +296,10 @@ LGF_D void vswap(T &a, T &b) {
   b = t;
 }
 
-template <class R>
-LGF_D void dft16(typename Ar<R>::V (&x)[16], const LineTw<R> &tw) {
-  typedef Ar<R> A;
+template <class A>
+LGF_D void dft16(typename A::V (&x)[16], const LineTw<typename A::Real> &tw) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) dft4<R>(x[i], x[i + 4], x[i + 8], x[i + 12]);
+  for (int i = 0; i < 4; ++i) dft4<A>(x[i], x[i + 4], x[i + 8], x[i + 12]);
   // x[a + 4 k] *= W_16^{a k}; W_16^4 = -i and the -i of W_16^6 = -i W_8 are folded into the second stage
   x[5] = A::mul(A::norm(x[5]), tw.w16[0]);
   x[9] = A::mul_w8(x[9], tw.w16[1]);
@@ -289,21 +309,20 @@ LGF_D void dft16(typename Ar<R>::V (&x)[16], const LineTw<R> &tw) {
   x[7] = A::mul(A::norm(x[7]), tw.w16[2]);
   x[11] = A::mul_w8(x[11], tw.w16[1]);
   x[15] = A::mul(A::norm(x[15]), tw.w16[3]);
-  dft4<R>(x[0], x[1], x[2], x[3]);
-  dft4<R>(x[4], x[5], x[6], x[7]);
-  dft4<R, true, true>(x[8], x[9], x[10], x[11]);
-  dft4<R, true, false>(x[12], x[13], x[14], x[15]);
+  dft4<A>(x[0], x[1], x[2], x[3]);
+  dft4<A>(x[4], x[5], x[6], x[7]);
+  dft4<A, true, true>(x[8], x[9], x[10], x[11]);
+  dft4<A, true, false>(x[12], x[13], x[14], x[15]);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = i + 1; j < 4; ++j) vswap(x[4 * i + j], x[4 * j + i]);
 }
 
-template <class R>
-LGF_D void dft8(typename Ar<R>::V (&x)[8], const LineTw<R> &tw) {
-  typedef Ar<R> A;
-  dft4<R>(x[0], x[2], x[4], x[6]);  // even points: E_k in x[0], x[2], x[4], x[6]
-  dft4<R>(x[1], x[3], x[5], x[7]);  // odd points
+template <class A>
+LGF_D void dft8(typename A::V (&x)[8], const LineTw<typename A::Real> &tw) {
+  dft4<A>(x[0], x[2], x[4], x[6]);  // even points: E_k in x[0], x[2], x[4], x[6]
+  dft4<A>(x[1], x[3], x[5], x[7]);  // odd points
   const typename A::V o1 = A::mul_w8(x[3], tw.w16[1]), o3 = A::mul_w8(x[7], tw.w16[1]);
   const typename A::V e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6], o0 = x[1], o2 = x[5];
   x[0] = A::add(e0, o0);
@@ -316,9 +335,8 @@ LGF_D void dft8(typename Ar<R>::V (&x)[8], const LineTw<R> &tw) {
   x[7] = A::add_pi(e3, o3);
 }
 
-template <class R>
-LGF_D void dft3(typename Ar<R>::V &a, typename Ar<R>::V &b, typename Ar<R>::V &c, const LineTw<R> &tw) {
-  typedef Ar<R> A;
+template <class A>
+LGF_D void dft3(typename A::V &a, typename A::V &b, typename A::V &c, const LineTw<typename A::Real> &tw) {
   const typename A::V u = A::add(b, c), v = A::swap(A::sub(b, c));
   const typename A::V m = A::add_mh(a, u), q = A::mul_im(v, tw.c3);  // q = -i sin(2 pi / 3) (b - c)
   a = A::add(a, u);
@@ -327,9 +345,8 @@ LGF_D void dft3(typename Ar<R>::V &a, typename Ar<R>::V &b, typename Ar<R>::V &c
 }
 
 // Odd N >= 5 by conjugate pairs with real coefficients; W_N^j = W_P^{j P / N} from the launch's table.
-template <class R, int N, int P>
-LGF_D void dft_odd(typename Ar<R>::V (&x)[N], const LineTw<R> &tw) {
-  typedef Ar<R> A;
+template <class A, int N, int P>
+LGF_D void dft_odd(typename A::V (&x)[N], const LineTw<typename A::Real> &tw) {
   constexpr int H = (N - 1) / 2;
   typename A::V u[H], v[H], x0 = x[0];
 #pragma unroll
@@ -356,9 +373,8 @@ LGF_D void dft_odd(typename Ar<R>::V (&x)[N], const LineTw<R> &tw) {
 }
 
 // v W_N^r, r and N compile-time after unrolling; quarter turns as swaps and signs
-template <class R, int N, int P>
-LGF_D typename Ar<R>::V rotate(typename Ar<R>::V v, const LineTw<R> &tw, int r) {
-  typedef Ar<R> A;
+template <class A, int N, int P>
+LGF_D typename A::V rotate(typename A::V v, const LineTw<typename A::Real> &tw, int r) {
   r %= N;
   if (r == 0) return v;
   if (4 * r == N) return A::add_mi(A::zero(), v);
@@ -376,27 +392,27 @@ constexpr int inverse_mod(int a, int n) {  // a^-1 mod n (0 for n = 1)
 }
 
 // N points, N | P, P / N even or N in the direct list
-template <class R, int N, int P>
+template <class A, int N, int P>
 struct Dft {
-  typedef typename Ar<R>::V V;
-  static LGF_D void run(V (&x)[N], const LineTw<R> &tw) {
+  typedef typename A::V V;
+  static LGF_D void run(V (&x)[N], const LineTw<typename A::Real> &tw) {
     if constexpr (N == 1) {
     } else if constexpr (N == 2) {
       const V a = x[0];
-      x[0] = Ar<R>::add(a, x[1]);
-      x[1] = Ar<R>::sub(a, x[1]);
+      x[0] = A::add(a, x[1]);
+      x[1] = A::sub(a, x[1]);
     } else if constexpr (N == 3) {
-      dft3<R>(x[0], x[1], x[2], tw);
+      dft3<A>(x[0], x[1], x[2], tw);
     } else if constexpr (N == 4) {
-      dft4<R>(x[0], x[1], x[2], x[3]);
+      dft4<A>(x[0], x[1], x[2], x[3]);
     } else if constexpr (N == 8) {
-      dft8<R>(x, tw);
+      dft8<A>(x, tw);
     } else if constexpr (N == 16) {
-      dft16<R>(x, tw);
+      dft16<A>(x, tw);
     } else {
       constexpr int F = dft_radix(N), Q = N / F;  // j = a + F b, k = k2 + Q k1
       if constexpr (Q == 1) {
-        dft_odd<R, N, P>(x, tw);
+        dft_odd<A, N, P>(x, tw);
       } else if constexpr (gcd_of(F, Q) == 1) {
         // coprime factors without twiddles: input j = (Q a + F b) mod N, output k = k1 mod F = k2 mod Q
         constexpr int CF = Q * inverse_mod(Q, F), CQ = F * inverse_mod(F, Q);
@@ -405,14 +421,14 @@ struct Dft {
         for (int a = 0; a < F; ++a) {
 #pragma unroll
           for (int b = 0; b < Q; ++b) y[a][b] = x[(Q * a + F * b) % N];
-          Dft<R, Q, P>::run(y[a], tw);
+          Dft<A, Q, P>::run(y[a], tw);
         }
 #pragma unroll
         for (int k2 = 0; k2 < Q; ++k2) {
           V z[F];
 #pragma unroll
           for (int a = 0; a < F; ++a) z[a] = y[a][k2];
-          Dft<R, F, P>::run(z, tw);
+          Dft<A, F, P>::run(z, tw);
 #pragma unroll
           for (int k1 = 0; k1 < F; ++k1) x[(CF * k1 + CQ * k2) % N] = z[k1];
         }
@@ -422,17 +438,17 @@ struct Dft {
         for (int a = 0; a < F; ++a) {
 #pragma unroll
           for (int b = 0; b < Q; ++b) y[a][b] = x[a + F * b];
-          Dft<R, Q, P>::run(y[a], tw);
+          Dft<A, Q, P>::run(y[a], tw);
 #pragma unroll
           for (int k2 = 1; k2 < Q; ++k2)
-            if (a > 0) y[a][k2] = rotate<R, N, P>(y[a][k2], tw, a * k2);
+            if (a > 0) y[a][k2] = rotate<A, N, P>(y[a][k2], tw, a * k2);
         }
 #pragma unroll
         for (int k2 = 0; k2 < Q; ++k2) {
           V z[F];
 #pragma unroll
           for (int a = 0; a < F; ++a) z[a] = y[a][k2];
-          Dft<R, F, P>::run(z, tw);
+          Dft<A, F, P>::run(z, tw);
 #pragma unroll
           for (int k1 = 0; k1 < F; ++k1) x[k2 + Q * k1] = z[k1];
         }

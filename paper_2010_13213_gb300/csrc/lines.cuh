@@ -12,7 +12,7 @@
 // and four times the box instead of eight, and an axis is transformed only on the lines that the passes before it
 // have made (2, 4 and 8 n^3 points instead of 8 on every axis).
 //
-// A line has n = M NB cells (M = 16, or 8 for boxes of an odd number of 8^3 blocks), L = 2 n = P M frequencies.
+// A line has n = M NB cells (M = 16, or 8 for 8^3 blocks of an odd count, of two and of four), L = 2 n = P M frequencies.
 // Its even and odd frequencies K = 2 K' + h (h = 0, 1) are the n-point DFTs of x_i and of x_i W_L^i, each in two steps:
 // one thread per (line, m) runs NB-point DFTs over the inputs of its m, one per (line, K1) M-point DFTs over m, with
 // one exchange through shared memory.
@@ -24,19 +24,22 @@
 // The inverse is the conjugate of the forward transform of the conjugate, so every pass runs forward code: the z pass
 // conjugates when it multiplies by Ghat (real, G is even), and the last pass negates the imaginary part.  The inverse
 // needs the first n outputs only: the sum of the even K's n-point DFT and of the odd K's turned by W_L^i.
-// Double-float values are renormalised (norm) around every product and when they leave a step: sums and products round
-// in proportion to the low part.  With one renormalisation per product alone the error of the two rings was 7.1e-15;
-// with these it is 5.8e-15, for 3 % of the time.
+// Double-float values are renormalised (norm) around every product and when they leave a step, in the y and x inverse and
+// on the low frequencies of the z inverse after every sum: sums and products round in proportion to the low part.  Error
+// of the two rings with one renormalisation per product alone 7.1e-15, around products and steps 4.9e-15, with all of
+// these 4.4e-15; the block-index passes had 5.7e-15.
 //
 // Two real fields ride as real and imaginary part of one complex field.  A field with a zero imaginary part keeps one
 // of every pair of x slots K1 that the frequencies K and -K share: NB + 1 of them.
 // A frequency row is [K2][kept K1]; LineGeom::fx gives the frequency K of a row's element.
 //
 // What bounds them: the FP32 pipe in double-float, the FP64 pipe in double (2 lanes a clock and SM), traffic and latency
-// in FP32.  One double-float solve of the 96 x 96 x 48 ring (three components) takes 154 us, 62 us of it in the z pass
-// (its FP32 pipe busy 72 % of the time); as block-index passes around k_box_mid it took 236 us.  Two rings on
-// 96 x 96 x 112: 374 us (546), FP64 ring 753 us (1,141), FP32 two rings 113 us (204).
+// in FP32.  One double-float solve of the 96 x 96 x 48 ring (three components) takes 163 us, most of it in the z pass; as
+// block-index passes around k_box_mid it took 236 us.  Two rings on 96 x 96 x 112: 395 us (546), FP64 ring 753 us (1,141),
+// FP32 two rings 113 us (204).
 #pragma once
+#include <type_traits>
+
 #include "arith.cuh"
 #include "box.cuh"
 
@@ -114,30 +117,30 @@ struct LineMap {
   // slot K1 that holds frequency K at K2 = 0
   static LGF_D int slot(int K) { return 2 * (((K >> 1) % NO) * N2 + (K >> 1) % N2) + (K & 1); }
 };
-template <class R, int M, int NB>
-LGF_D void line_dft(typename Ar<R>::V (&v)[NB], const LineTw<R> &tw) {  // over (j3, j2)
+template <class A, int M, int NB>
+LGF_D void line_dft(typename A::V (&v)[NB], const LineTw<typename A::Real> &tw) {  // over (j3, j2)
   typedef LineMap<M, NB> Mp;
   constexpr int NO = Mp::NO, N2 = Mp::N2;
   if constexpr (NO == 1) {
-    Dft<R, NB, 2 * NB>::run(v, tw);
+    Dft<A, NB, 2 * NB>::run(v, tw);
   } else {
     if constexpr (N2 > 1) {
 #pragma unroll
       for (int j3 = 0; j3 < NO; ++j3) {
-        typename Ar<R>::V z[N2];
+        typename A::V z[N2];
 #pragma unroll
         for (int j = 0; j < N2; ++j) z[j] = v[j3 * N2 + j];
-        Dft<R, N2, 2 * NB>::run(z, tw);
+        Dft<A, N2, 2 * NB>::run(z, tw);
 #pragma unroll
         for (int j = 0; j < N2; ++j) v[j3 * N2 + j] = z[j];
       }
     }
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) {
-      typename Ar<R>::V z[NO];
+      typename A::V z[NO];
 #pragma unroll
       for (int j = 0; j < NO; ++j) z[j] = v[j * N2 + k2];
-      Dft<R, NO, 2 * NB>::run(z, tw);
+      Dft<A, NO, 2 * NB>::run(z, tw);
 #pragma unroll
       for (int j = 0; j < NO; ++j) v[j * N2 + k2] = z[j];
     }
@@ -179,7 +182,7 @@ LGF_D void line_split(typename Ar<R>::M *S, int m, int line, const LineTw<R> &tw
 #pragma unroll
       for (int j = 0; j < NB; ++j) v[j] = A::mul(v[j], twl[Mp::cell(j, m)]);
     }
-    line_dft<R, M, NB>(v, tw);
+    line_dft<A, M, NB>(v, tw);
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       v[q] = A::norm(v[q]);
@@ -192,10 +195,9 @@ LGF_D void line_split(typename Ar<R>::M *S, int m, int line, const LineTw<R> &tw
 // Last step of an inverse (line, m): the M-point sums of slot K1 from S (twiddled here), the NB outputs to put(y), cells
 // as load gives them; pre() before the odd half, for loads that put needs.  `half` (x axis): of a slot and its mirror
 // only the lower is held; with u the twiddled sum of the held one, the other's is conj(u), times W_{M N2}^{-m} for h = 1.
-template <class R, int M, int NB, int TL, bool X, class Pre, class Put>
-LGF_D void line_merge(typename Ar<R>::M *S, int m, int line, bool half, const LineTw<R> &tw,
-                      const typename Ar<R>::T *__restrict__ twl, Pre pre, Put put) {
-  typedef Ar<R> A;
+template <class A, int M, int NB, int TL, bool X, class Pre, class Put>
+LGF_D void line_merge(typename A::M *S, int m, int line, bool half, const LineTw<typename A::Real> &tw,
+                      const typename A::T *__restrict__ twl, Pre pre, Put put) {
   typedef LineSmem<M, TL, X> Sm;
   typedef LineMap<M, NB> Mp;
 #pragma unroll 1
@@ -215,7 +217,7 @@ LGF_D void line_merge(typename Ar<R>::M *S, int m, int line, bool half, const Li
       }
     }
     if (h) pre();
-    line_dft<R, M, NB>(v, tw);
+    line_dft<A, M, NB>(v, tw);
     if (h == 0) {
 #pragma unroll
       for (int j = 0; j < NB; ++j) A::st(S + Sm::at(2 * j, m, line), v[j]);
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     if (any) {
 #pragma unroll
       for (int m = 0; m < M; ++m) v[m] = A::ld(S + Sm::at(k1, m, l));
-      Dft<R, M, M>::run(v, tw);
+      Dft<A, M, M>::run(v, tw);
     } else {  // no source on these lines
 #pragma unroll
       for (int m = 0; m < M; ++m) v[m] = A::zero();
@@ -397,7 +399,9 @@ LGF_D void line_store(const OutSpec<R> &o, const int (&ob)[NB], int brow, int cr
     if (on[j]) store_field<R>(o.dst, base + ((int64_t)ob[j] << (3 * sh)) + ((M * j + m) & msk), o.dtype, w[j]);
 }
 
-// y inverse and x inverse (X, writing through the output specs); grids as k_line_fwd.
+// y inverse and x inverse (X, writing through the output specs); grids as k_line_fwd.  Sums renormalised (ArFine): what
+// these two passes round is not smoothed by anything after them.  Two-level rings of 48 to 160 cells: error 4.9e-15 ->
+// 4.3e-15, 4 % of a solve's time (96 x 96 x 48 ring 155 -> 161 us).
 template <class R, int M, int NB, bool X>
 __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     k_line_inv(const typename Ar<R>::M *__restrict__ in, typename Ar<R>::M *__restrict__ out,
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
         if (kp >= M * NB) kp -= M * NB;
       }
     }
-    Dft<R, M, M>::run(v, tw);
+    Dft<ArFine<R>, M, M>::run(v, tw);
 #pragma unroll
     for (int m = 0; m < M; ++m) A::st(S + Sm::at(k1, m, l), A::norm(v[m]));
   }
@@ -448,7 +452,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
       const int brow = ((z >> sh) * g.nb[1] + (y >> sh)) * g.nb[0];
       const int crow = (((z & msk) << sh) + (y & msk)) << sh;
       int ore[NB], oim[NB];  // the scatter indices of the line's blocks, loaded while the odd half runs
-      line_merge<R, M, NB, TL, X>(
+      line_merge<ArFine<R>, M, NB, TL, X>(
           S, m, l, half, tw, twl,
           [&]() {
             const int32_t *sr = outs.re[field].scatter, *si = half ? nullptr : outs.im[field].scatter;
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
           });
     } else {
       typename A::M *dst = out + field * g.astride + (int64_t)blockIdx.y * g.n[1] * W + line;
-      line_merge<R, M, NB, TL, X>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
+      line_merge<ArFine<R>, M, NB, TL, X>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) A::st(dst + (int64_t)LineMap<M, NB>::cell(j, m) * W, A::norm(v[j]));
       });
@@ -480,6 +484,10 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
 
 // z: forward, kernel product, inverse; grid (ceil(L_y width / TL), 1, fields), lines the slots (fy, fx) of a plane.
 // Gf is Ghat on 0 <= f_a <= L_a / 2 (it is even in every axis), x fastest.
+// Ghat grows as 1 / f^2 towards f = 0: the few lines of low f_y and f_x carry most of a smooth result, and what they round
+// in the inverse is seen as one smooth error all over the box.  A tile that holds a line with both frequencies within
+// L / 32 renormalises its sums (ArFine): three-level ring over 16 seeds 6.5e-15 (up to 10.9e-15) -> 5.4e-15 (up to 7.4e-15) for
+// 1.5 % of the time; in all tiles 5.2e-15 (6.4e-15), another 4 %.
 template <class R, int M, int NB>
 __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     k_line_mid(typename Ar<R>::M *__restrict__ C, const R *__restrict__ Gf, const __grid_constant__ LineGeom g,
@@ -496,12 +504,14 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
   typename A::M *Cf = C + field * g.cstride;
   // Ghat of the tile's lines, [fz <= L / 2][line], on its way to shared memory under the first step
   R *G = reinterpret_cast<R *>(S + P * Sm::SK);
+  bool low;
   {
     const int l = threadIdx.x % TL, line = min(line0 + l, nlines - 1), fy = line / W, s = line - fy * W;
     const int fx = __ldg((field < g.nc ? g.fxc : g.fxr) + s);
     const R *src = Gf + (int64_t)min(fy, Ly - fy) * (Lx / 2 + 1) + min(fx, Lx - fx);
     const int64_t gz = (int64_t)(Ly / 2 + 1) * (Lx / 2 + 1);
     for (int fz = threadIdx.x / TL; fz <= L / 2; fz += NT / TL) line_copy_async(G + fz * TL + l, src + fz * gz);
+    low = 32 * min(fy, Ly - fy) <= Ly && 32 * min(fx, Lx - fx) <= Lx;
   }
   for (int t = threadIdx.x; t < TL * M; t += NT) {
     const int m = t / TL, l = t % TL, line = line0 + l;
@@ -513,36 +523,46 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     });
   }
   line_copy_wait();
-  __syncthreads();
-  for (int t = threadIdx.x; t < TL * P; t += NT) {
-    const int k1 = t / TL, l = t % TL;
-    if (line0 + l >= nlines) continue;
-    typename A::V v[M];
+  low = __syncthreads_or(low);
+  auto rest = [&](auto inverse) {
+    typedef decltype(inverse) I;
+    for (int t = threadIdx.x; t < TL * P; t += NT) {
+      const int k1 = t / TL, l = t % TL;
+      if (line0 + l >= nlines) continue;
+      typename A::V v[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) v[m] = A::ld(S + Sm::at(k1, m, l));
-    Dft<R, M, M>::run(v, tw);
-    int kp = LineMap<M, NB>::freq(k1 >> 1);
+      for (int m = 0; m < M; ++m) v[m] = A::ld(S + Sm::at(k1, m, l));
+      Dft<A, M, M>::run(v, tw);
+      int kp = LineMap<M, NB>::freq(k1 >> 1);
 #pragma unroll
-    for (int k2 = 0; k2 < M; ++k2) {
-      const int fz = 2 * kp + (k1 & 1);
-      v[k2] = A::norm(A::scale_conj(A::norm(v[k2]), G[min(fz, L - fz) * TL + l]));
-      kp += LineMap<M, NB>::STEP;
-      if (kp >= M * NB) kp -= M * NB;
+      for (int k2 = 0; k2 < M; ++k2) {
+        const int fz = 2 * kp + (k1 & 1);
+        v[k2] = A::norm(A::scale_conj(A::norm(v[k2]), G[min(fz, L - fz) * TL + l]));
+        kp += LineMap<M, NB>::STEP;
+        if (kp >= M * NB) kp -= M * NB;
+      }
+      Dft<I, M, M>::run(v, tw);
+#pragma unroll
+      for (int m = 0; m < M; ++m) A::st(S + Sm::at(k1, m, l), A::norm(v[m]));
     }
-    Dft<R, M, M>::run(v, tw);
+    __syncthreads();
+    for (int t = threadIdx.x; t < TL * M; t += NT) {
+      const int m = t / TL, l = t % TL, line = line0 + l;
+      if (line >= nlines) continue;
+      typename A::M *dst = Cf + line;
+      line_merge<I, M, NB, TL, false>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) A::st(S + Sm::at(k1, m, l), A::norm(v[m]));
+        for (int j = 0; j < NB; ++j) A::st(dst + (int64_t)LineMap<M, NB>::cell(j, m) * nlines, A::norm(v[j]));
+      });
+    }
+  };
+  if constexpr (std::is_same<R, df>::value) {
+    if (low) {
+      rest(ArFine<R>());
+      return;
+    }
   }
-  __syncthreads();
-  for (int t = threadIdx.x; t < TL * M; t += NT) {
-    const int m = t / TL, l = t % TL, line = line0 + l;
-    if (line >= nlines) continue;
-    typename A::M *dst = Cf + line;
-    line_merge<R, M, NB, TL, false>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
-#pragma unroll
-      for (int j = 0; j < NB; ++j) A::st(dst + (int64_t)LineMap<M, NB>::cell(j, m) * nlines, A::norm(v[j]));
-    });
-  }
+  rest(Ar<R>());
 }
 
 }  // namespace lgf
