@@ -155,6 +155,10 @@ struct BoxSpec {
   ~BoxSpec();
 };
 
+// The end of a plan's uploads (cudaMemcpy from pageable memory on the legacy stream), before any other stream can use them:
+// such a copy may return before the transfer has ended, and the caller's streams do not wait for the legacy stream.
+inline bool uploads_ended() { return cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess; }
+
 // Growable device buffer (never shrinks; freed with the owner).
 struct DevBuf {
   void *p = nullptr;

@@ -416,6 +416,11 @@ int build_plan(const lgf_mesh *m, const int *heat_radii, Plan **out) {
       return rc;
     }
   }
+  if (!uploads_ended()) {
+    cudaGetLastError();
+    delete P;
+    return set_error(LGF_E_CUDA, "plan upload failed");
+  }
   *out = P;
   return LGF_OK;
 }

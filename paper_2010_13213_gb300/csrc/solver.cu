@@ -156,10 +156,16 @@ static int single_plan(const lgf_mesh *m, SinglePlan **out) {
     delete P;
     return set_error(LGF_E_OOM, "single-level plan allocation failed");
   }
-  if (!idx.empty()) cudaMemcpy(P->d_idx, idx.data(), sizeof(int32_t) * idx.size(), cudaMemcpyHostToDevice);
-  if (!cs.empty()) cudaMemcpy(P->d_c, cs.data(), sizeof(int4) * cs.size(), cudaMemcpyHostToDevice);
-  if (!tmap.empty()) cudaMemcpy(P->d_tmap, tmap.data(), sizeof(int32_t) * tmap.size(), cudaMemcpyHostToDevice);
-  if (!is_src.empty()) cudaMemcpy(P->d_is_src, is_src.data(), is_src.size(), cudaMemcpyHostToDevice);
+  auto up = [](void *dst, const void *src, size_t bytes) {
+    return !bytes || cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+  };
+  if (!up(P->d_idx, idx.data(), sizeof(int32_t) * idx.size()) || !up(P->d_c, cs.data(), sizeof(int4) * cs.size()) ||
+      !up(P->d_tmap, tmap.data(), sizeof(int32_t) * tmap.size()) || !up(P->d_is_src, is_src.data(), is_src.size()) ||
+      !uploads_ended()) {
+    cudaGetLastError();
+    delete P;
+    return set_error(LGF_E_CUDA, "single-level plan upload failed");
+  }
   g_sp.emplace_front(key, P);
   while (g_sp.size() > 1024) {
     delete g_sp.back().second;
