@@ -504,14 +504,14 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
   typename A::M *Cf = C + field * g.cstride;
   // Ghat of the tile's lines, [fz <= L / 2][line], on its way to shared memory under the first step
   R *G = reinterpret_cast<R *>(S + P * Sm::SK);
-  bool low;
+  bool low = false;
   {
     const int l = threadIdx.x % TL, line = min(line0 + l, nlines - 1), fy = line / W, s = line - fy * W;
     const int fx = __ldg((field < g.nc ? g.fxc : g.fxr) + s);
     const R *src = Gf + (int64_t)min(fy, Ly - fy) * (Lx / 2 + 1) + min(fx, Lx - fx);
     const int64_t gz = (int64_t)(Ly / 2 + 1) * (Lx / 2 + 1);
     for (int fz = threadIdx.x / TL; fz <= L / 2; fz += NT / TL) line_copy_async(G + fz * TL + l, src + fz * gz);
-    low = 32 * min(fy, Ly - fy) <= Ly && 32 * min(fx, Lx - fx) <= Lx;
+    if constexpr (std::is_same<R, df>::value) low = 32 * min(fy, Ly - fy) <= Ly && 32 * min(fx, Lx - fx) <= Lx;
   }
   for (int t = threadIdx.x; t < TL * M; t += NT) {
     const int m = t / TL, l = t % TL, line = line0 + l;
@@ -523,7 +523,8 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     });
   }
   line_copy_wait();
-  low = __syncthreads_or(low);
+  if constexpr (std::is_same<R, df>::value) low = __syncthreads_or(low);
+  else __syncthreads();
   auto rest = [&](auto inverse) {
     typedef decltype(inverse) I;
     for (int t = threadIdx.x; t < TL * P; t += NT) {
