@@ -69,10 +69,12 @@ struct BoxOps {
   // group of fields (phase timing; may be null).  `slices` > 0 runs the block-index DFTs as tensor-core GEMMs
   // with that many BF16 digit slices (float: 1-3, double-float: 4-6) around k_box_mid; a bounded wait that
   // gives up there sets *status.  `blocks` (FP32): the block-index passes of box_pass.cuh instead of the line passes.
+  // `fine`: the result is differenced (LineFine in lines.cuh).
   static int convolve(int B, const BoxSpec *S, int nf, const int *nin, const InSpec3 *in,
                       const OutSpec<R> *ore, const OutSpec<R> *oim, double scale, cx<R> *Y0, cx<R> *Y1,
                       cudaStream_t st, void (*mark)(void *, int) = nullptr, void *mark_ctx = nullptr,
-                      int slices = 0, bool blocks = false, int *status = nullptr, int64_t *launches = nullptr);
+                      int slices = 0, bool blocks = false, int *status = nullptr, int64_t *launches = nullptr,
+                      bool fine = false);
 };
 
 // Launch of one tensor-core pass: persistent CTAs of 128 threads, as many per SM as registers, shared
@@ -311,7 +313,7 @@ static int box_group_blocks(const BoxSpec *S, const std::vector<int> &fields, in
 template <class R>
 static int box_group_lines(int B, const BoxSpec *S, const std::vector<int> &fields, int nc, const int *nin,
                            const InSpec3 *in, const OutSpec<R> *ore, const OutSpec<R> *oim, double scale, cx<R> *Y0,
-                           cx<R> *Y1, cudaStream_t st, void (*mark)(void *, int), void *mark_ctx) {
+                           cx<R> *Y1, cudaStream_t st, void (*mark)(void *, int), void *mark_ctx, bool fine) {
   typedef typename Ar<R>::M M;
   static_assert(sizeof(M) == sizeof(cx<R>), "the scratch is sized in complex values");
   LinePass<R> p;
@@ -345,6 +347,7 @@ static int box_group_lines(int B, const BoxSpec *S, const std::vector<int> &fiel
   p.nfields = n;
   p.wmax = nc > 0 ? g.wc : g.wr;
   p.scale = scale;
+  p.fine = fine;
   p.st = st;
   M *A = (M *)Y0, *C = (M *)Y1;
   bool ok = true;
@@ -371,7 +374,7 @@ template <class R>
 int BoxOps<R>::convolve(int B, const BoxSpec *S, int nf, const int *nin, const InSpec3 *in,
                         const OutSpec<R> *ore, const OutSpec<R> *oim, double scale, cx<R> *Y0, cx<R> *Y1,
                         cudaStream_t st, void (*mark)(void *, int), void *mark_ctx, int slices, bool blocks, int *status,
-                        int64_t *launches) {
+                        int64_t *launches, bool fine) {
   if (slices > 0 && (std::is_same<R, double>::value || !status))
     return set_error(LGF_E_UNSUPPORTED, "the tensor-core DFT-GEMM runs in FP32 or double-float only");
   if (B != 8 && B != 16) return set_error(LGF_E_UNSUPPORTED, "block size %d", B);
@@ -401,7 +404,7 @@ int BoxOps<R>::convolve(int B, const BoxSpec *S, int nf, const int *nin, const I
         // the double-float Ghat carries the rest of the 1 / (8 cells) of the inverse transform
         rc = box_group_lines<R>(B, S, grp, nc, nin, in, ore, oim,
                                 scale / (std::is_same<R, df>::value ? box_pow2((int64_t)cells8) : cells8), Y0, Y1, st, mark,
-                                mark_ctx);
+                                mark_ctx, fine);
       } else if constexpr (!std::is_same<R, double>::value) {
         rc = B == 8 ? box_group_blocks<R, 8>(S, grp, nc, nin, in, ore, oim, scale / cells8, Y0, Y1, st, mark, mark_ctx,
                                              slices, status)

@@ -19,11 +19,12 @@ struct LinePass {
   const R *Gf = nullptr;
   double scale = 1.0;
   int nfields = 0, wmax = 0;              // fields of the launch, their widest frequency row
+  bool fine = false;                      // renormalised sums where the shape has them (LineFine)
   cudaStream_t st = nullptr;
 };
 
-template <class R, int M, int NB>
-void line_launch(LineKind kind, const LinePass<R> &p) {
+template <class R, int M, int NB, bool FINE>
+void line_launch_as(LineKind kind, const LinePass<R> &p) {
   constexpr int TL = LineTile<M, NB>::TL, NT = LineTile<M, NB>::NT;
   constexpr size_t smx = line_smem<R, M, NB, true>(), smy = line_smem<R, M, NB, false>(),
                    smm = line_smem_mid<R, M, NB>();
@@ -41,21 +42,28 @@ void line_launch(LineKind kind, const LinePass<R> &p) {
       break;
     case LINE_MID: {
       const unsigned tiles = (unsigned)(((int64_t)p.g.P[1] * p.g.M[1] * p.wmax + TL - 1) / TL);
-      smem_limit(done[kind], k_line_mid<R, M, NB>, smm);
-      k_line_mid<R, M, NB><<<dim3(tiles, 1, nf), NT, smm, p.st>>>(p.out, p.Gf, p.g, *p.tw, p.twl);
+      smem_limit(done[kind], k_line_mid<R, M, NB, FINE>, smm);
+      k_line_mid<R, M, NB, FINE><<<dim3(tiles, 1, nf), NT, smm, p.st>>>(p.out, p.Gf, p.g, *p.tw, p.twl);
       break;
     }
     case LINE_INV_Y:
-      smem_limit(done[kind], k_line_inv<R, M, NB, false>, smy);
-      k_line_inv<R, M, NB, false><<<dim3(tiles_w, nz, nf), NT, smy, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
-                                                                           1.0);
+      smem_limit(done[kind], k_line_inv<R, M, NB, false, FINE>, smy);
+      k_line_inv<R, M, NB, false, FINE><<<dim3(tiles_w, nz, nf), NT, smy, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
+                                                                                 1.0);
       break;
     case LINE_INV_X:
-      smem_limit(done[kind], k_line_inv<R, M, NB, true>, smx);
-      k_line_inv<R, M, NB, true><<<dim3(tiles_yz, 1, nf), NT, smx, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
-                                                                          p.scale);
+      smem_limit(done[kind], k_line_inv<R, M, NB, true, FINE>, smx);
+      k_line_inv<R, M, NB, true, FINE><<<dim3(tiles_yz, 1, nf), NT, smx, p.st>>>(p.in, p.out, p.g, *p.tw, p.twl, *p.outs,
+                                                                                p.scale);
       break;
   }
+}
+template <class R, int M, int NB>
+void line_launch(LineKind kind, const LinePass<R> &p) {
+  if constexpr (LineFine<R, M>::value) {
+    if (p.fine) return line_launch_as<R, M, NB, true>(kind, p);
+  }
+  line_launch_as<R, M, NB, false>(kind, p);
 }
 
 // The pass for NB in [LO, HI] (steps of ST); one translation unit per range and arithmetic.

@@ -24,19 +24,19 @@
 // The inverse is the conjugate of the forward transform of the conjugate, so every pass runs forward code: the z pass
 // conjugates when it multiplies by Ghat (real, G is even), and the last pass negates the imaginary part.  The inverse
 // needs the first n outputs only: the sum of the even K's n-point DFT and of the odd K's turned by W_L^i.
-// Double-float values are renormalised (norm) around every product and when they leave a step, in the y and x inverse and
-// on the low frequencies of the z inverse after every sum: sums and products round in proportion to the low part.  Error
-// of the two rings with one renormalisation per product alone 7.1e-15, around products and steps 4.9e-15, with all of
-// these 4.4e-15; the block-index passes had 5.7e-15.
+// Double-float values are renormalised (norm) around every product and when they leave a step: sums and products round
+// in proportion to the low part.  With one renormalisation per product alone the error of the two rings was 7.1e-15;
+// with these it is 4.9e-15, for 3 % of the time; the block-index passes had 5.7e-15.  Where a result is differenced the
+// inverse passes also renormalise after every sum (LineFine).
 //
 // Two real fields ride as real and imaginary part of one complex field.  A field with a zero imaginary part keeps one
 // of every pair of x slots K1 that the frequencies K and -K share: NB + 1 of them.
 // A frequency row is [K2][kept K1]; LineGeom::fx gives the frequency K of a row's element.
 //
 // What bounds them: the FP32 pipe in double-float, the FP64 pipe in double (2 lanes a clock and SM), traffic and latency
-// in FP32.  One double-float solve of the 96 x 96 x 48 ring (three components) takes 163 us, most of it in the z pass; as
-// block-index passes around k_box_mid it took 236 us.  Two rings on 96 x 96 x 112: 395 us (546), FP64 ring 753 us (1,141),
-// FP32 two rings 113 us (204).
+// in FP32.  One double-float solve of the 96 x 96 x 48 ring (three components) takes 154 us, 62 us of it in the z pass
+// (its FP32 pipe busy 72 % of the time); as block-index passes around k_box_mid it took 236 us.  Two rings on
+// 96 x 96 x 112: 374 us (546), FP64 ring 753 us (1,141), FP32 two rings 113 us (204).
 #pragma once
 #include <type_traits>
 
@@ -76,6 +76,17 @@ struct LineGeom {
   int wc, wr;             // frequency row length of a complex and of a real field
   const int32_t *fxc, *fxr;  // x frequency of a row's element, complex and real fields
   int64_t astride, cstride;  // field strides of A and C
+};
+// Line shapes whose inverse and z kernels have a form with renormalised sums (FINE, ArFine): double-float in 16-point
+// steps.  It serves composite solves and the velocity refresh, which difference the result (corrections, the curl).  With
+// lazy sums composite solves on 16^3 blocks had 1.15 times the error of the block-index passes (mean of 24 meshes, up to
+// 1.5 times) and have 0.99 times now, refreshes of a few blocks 1.28 and 1.15; plain solves have 0.81 times with lazy sums
+// and keep them.  Three-level ring 4.45 -> 4.68 ms, refresh of 6 x 6 x 3 blocks 311 -> 324 us.  Lines in 8-point steps come
+// from 8^3 blocks, where lazy sums have 0.45 to 0.85 times that error in composite solves too (5 x 7 x 3 blocks with
+// renormalised sums: 36.9 -> 40.5 us).
+template <class R, int M>
+struct LineFine {
+  static constexpr bool value = std::is_same<R, df>::value && M == 16;
 };
 LGF_HD int line_width(const LineGeom &g, int field) { return field < g.nc ? g.wc : g.wr; }
 
@@ -399,15 +410,16 @@ LGF_D void line_store(const OutSpec<R> &o, const int (&ob)[NB], int brow, int cr
     if (on[j]) store_field<R>(o.dst, base + ((int64_t)ob[j] << (3 * sh)) + ((M * j + m) & msk), o.dtype, w[j]);
 }
 
-// y inverse and x inverse (X, writing through the output specs); grids as k_line_fwd.  Sums renormalised (ArFine): what
-// these two passes round is not smoothed by anything after them.  Two-level rings of 48 to 160 cells: error 4.9e-15 ->
-// 4.3e-15, 4 % of a solve's time (96 x 96 x 48 ring 155 -> 161 us).
-template <class R, int M, int NB, bool X>
+// y inverse and x inverse (X, writing through the output specs); grids as k_line_fwd.  Fine: all sums renormalised, as what
+// these two passes round is not smoothed by anything after them (two-level rings of 48 to 160 cells: error 4.9e-15 ->
+// 4.3e-15 for 4 % of the time).
+template <class R, int M, int NB, bool X, bool FINE>
 __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     k_line_inv(const typename Ar<R>::M *__restrict__ in, typename Ar<R>::M *__restrict__ out,
                const __grid_constant__ LineGeom g, const __grid_constant__ LineTw<R> tw,
                const typename Ar<R>::T *__restrict__ twl, const __grid_constant__ InvOuts<R> outs, double scale) {
   typedef Ar<R> A;
+  typedef std::conditional_t<FINE, ArFine<R>, Ar<R>> I;
   constexpr int NT = LineTile<M, NB>::NT, TL = LineTile<M, NB>::TL, P = 2 * NB;
   typedef LineSmem<M, TL, X> Sm;
   extern __shared__ __align__(16) unsigned char line_smem_raw[];
@@ -437,7 +449,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
         if (kp >= M * NB) kp -= M * NB;
       }
     }
-    Dft<ArFine<R>, M, M>::run(v, tw);
+    Dft<I, M, M>::run(v, tw);
 #pragma unroll
     for (int m = 0; m < M; ++m) A::st(S + Sm::at(k1, m, l), A::norm(v[m]));
   }
@@ -452,7 +464,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
       const int brow = ((z >> sh) * g.nb[1] + (y >> sh)) * g.nb[0];
       const int crow = (((z & msk) << sh) + (y & msk)) << sh;
       int ore[NB], oim[NB];  // the scatter indices of the line's blocks, loaded while the odd half runs
-      line_merge<ArFine<R>, M, NB, TL, X>(
+      line_merge<I, M, NB, TL, X>(
           S, m, l, half, tw, twl,
           [&]() {
             const int32_t *sr = outs.re[field].scatter, *si = half ? nullptr : outs.im[field].scatter;
@@ -474,7 +486,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
           });
     } else {
       typename A::M *dst = out + field * g.astride + (int64_t)blockIdx.y * g.n[1] * W + line;
-      line_merge<ArFine<R>, M, NB, TL, X>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
+      line_merge<I, M, NB, TL, X>(S, m, l, false, tw, twl, []() {}, [&](typename A::V (&v)[NB]) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) A::st(dst + (int64_t)LineMap<M, NB>::cell(j, m) * W, A::norm(v[j]));
       });
@@ -485,10 +497,10 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
 // z: forward, kernel product, inverse; grid (ceil(L_y width / TL), 1, fields), lines the slots (fy, fx) of a plane.
 // Gf is Ghat on 0 <= f_a <= L_a / 2 (it is even in every axis), x fastest.
 // Ghat grows as 1 / f^2 towards f = 0: the few lines of low f_y and f_x carry most of a smooth result, and what they round
-// in the inverse is seen as one smooth error all over the box.  A tile that holds a line with both frequencies within
-// L / 32 renormalises its sums (ArFine): three-level ring over 16 seeds 6.5e-15 (up to 10.9e-15) -> 5.4e-15 (up to 7.4e-15) for
-// 1.5 % of the time; in all tiles 5.2e-15 (6.4e-15), another 4 %.
-template <class R, int M, int NB>
+// in the inverse is seen as one smooth error all over the box.  Fine: a tile that holds a line with both frequencies within
+// L / 32 renormalises its sums (three-level ring over 16 seeds, beside fine y and x passes: 6.5e-15, up to 10.9e-15 ->
+// 5.4e-15, up to 7.4e-15, for 1.5 % of the time; in all tiles 5.2e-15 and 6.4e-15 for another 4 %).
+template <class R, int M, int NB, bool FINE>
 __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     k_line_mid(typename Ar<R>::M *__restrict__ C, const R *__restrict__ Gf, const __grid_constant__ LineGeom g,
                const __grid_constant__ LineTw<R> tw, const typename Ar<R>::T *__restrict__ twl) {
@@ -511,7 +523,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     const R *src = Gf + (int64_t)min(fy, Ly - fy) * (Lx / 2 + 1) + min(fx, Lx - fx);
     const int64_t gz = (int64_t)(Ly / 2 + 1) * (Lx / 2 + 1);
     for (int fz = threadIdx.x / TL; fz <= L / 2; fz += NT / TL) line_copy_async(G + fz * TL + l, src + fz * gz);
-    if constexpr (std::is_same<R, df>::value) low = 32 * min(fy, Ly - fy) <= Ly && 32 * min(fx, Lx - fx) <= Lx;
+    if constexpr (FINE) low = 32 * min(fy, Ly - fy) <= Ly && 32 * min(fx, Lx - fx) <= Lx;
   }
   for (int t = threadIdx.x; t < TL * M; t += NT) {
     const int m = t / TL, l = t % TL, line = line0 + l;
@@ -523,7 +535,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
     });
   }
   line_copy_wait();
-  if constexpr (std::is_same<R, df>::value) low = __syncthreads_or(low);
+  if constexpr (FINE) low = __syncthreads_or(low);
   else __syncthreads();
   auto rest = [&](auto inverse) {
     typedef decltype(inverse) I;
@@ -557,7 +569,7 @@ __global__ void __launch_bounds__(LineTile<M, NB>::NT, LineTile<M, NB>::MB)
       });
     }
   };
-  if constexpr (std::is_same<R, df>::value) {
+  if constexpr (FINE) {
     if (low) {
       rest(ArFine<R>());
       return;

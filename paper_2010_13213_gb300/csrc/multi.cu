@@ -315,7 +315,7 @@ static int solve_multi_t(lgf_table *t, const lgf_mesh *m, int ncomp, const void 
       const int nf = (int)nin.size();
       if ((rc = BoxOps<R>::convolve(B, S, nf, nin.data(), in.data(), ore.data(), oim.data(), scale, Y0, Y1, st,
                                     o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, box_blocks(o, dtype),
-                                    t->d_status, &launches)))
+                                    t->d_status, &launches, K > 1)))
         return rc;
       target_cells += L.n_omega;
       nsrc_total += nSA + nSB;

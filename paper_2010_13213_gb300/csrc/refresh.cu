@@ -156,7 +156,7 @@ extern "C" int lgf_velocity_refresh(lgf_table *t, const lgf_mesh *m, const void 
   for (int c = 0; c < 3; ++c)
     cudaMemcpyAsync((char *)om + es * c * ext_cs, (const char *)omega_dev + es * c * ucs, es * ucs,
                     cudaMemcpyDeviceToDevice, st);
-  rc = solve_poisson(t, &me, 3, om, psi, dtype, o, rep, st);
+  rc = solve_poisson(t, &me, 3, om, psi, dtype, o, rep, st, true);
   if (rc == LGF_OK) {
     const double inv_h = 1.0 / m->h0;
     if (dtype == LGF_F64)

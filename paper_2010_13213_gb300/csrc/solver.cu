@@ -259,7 +259,7 @@ static size_t dtype_size(int dtype, size_t rsize) { return dtype == 0 ? 8 : (dty
 
 template <class R>
 static int solve_single_box(lgf_table *t, const lgf_mesh *m, const SinglePlan *P, int ncomp, const void *f,
-                            void *phi, int dtype, const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st) {
+                            void *phi, int dtype, const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st, bool fine) {
   const int B = m->block, n = m->nblocks[0];
   const int64_t B3 = (int64_t)B * B * B;
   BoxSpec *S = nullptr;
@@ -291,7 +291,7 @@ static int solve_single_box(lgf_table *t, const lgf_mesh *m, const SinglePlan *P
   if ((rc = BoxOps<R>::convolve(B, S, nf, nin.data(), in.data(), ore.data(), oim.data(), scale,
                                 (cx<R> *)ws->buf[0].p, (cx<R> *)ws->buf[1].p, st,
                                 o.timing ? phase_mark_cb : nullptr, &tm, o.dft_slices, box_blocks(o, dtype),
-                                t->d_status, &launches)))
+                                t->d_status, &launches, fine)))
     return rc;
   tm.finish(rep);
   fill_report(rep, P, B3, ws, launches, LGF_MAC_BOX, (int64_t)S->bytes);
@@ -340,7 +340,7 @@ static int single_residual(lgf_table *t, const lgf_mesh *m, const SinglePlan *P,
 
 template <class R>
 static int solve_single_any(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, void *phi, int dtype,
-                            const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st) {
+                            const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st, bool fine) {
   SinglePlan *P = nullptr;
   int rc = single_plan(m, &P);
   if (rc) return rc;
@@ -353,7 +353,7 @@ static int solve_single_any(lgf_table *t, const lgf_mesh *m, int ncomp, const vo
                : LGF_MAC_PAIR;
   if (mode == LGF_MAC_BOX) {
     if (!P->box_ok) return set_error(LGF_E_UNSUPPORTED, "BOX mode needs 1..%d blocks per axis", BOX_NB_MAX);
-    rc = solve_single_box<R>(t, m, P, ncomp, f, phi, dtype, o, rep, st);
+    rc = solve_single_box<R>(t, m, P, ncomp, f, phi, dtype, o, rep, st, fine);
   } else {
     rc = solve_single_pair<R>(t, m, P, ncomp, f, phi, dtype, o, rep, st);
   }
@@ -362,12 +362,12 @@ static int solve_single_any(lgf_table *t, const lgf_mesh *m, int ncomp, const vo
 }
 
 int solve_poisson(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, void *phi, int dtype,
-                  const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st) {
+                  const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st, bool fine) {
   if (m->nlevels > 1) return solve_multi(t, m, ncomp, f, phi, dtype, o, rep, st, nullptr);
   switch (o.precision) {
-    case LGF_PREC_FP64: return solve_single_any<double>(t, m, ncomp, f, phi, dtype, o, rep, st);
-    case LGF_PREC_FP32: return solve_single_any<float>(t, m, ncomp, f, phi, dtype, o, rep, st);
-    default: return solve_single_any<df>(t, m, ncomp, f, phi, dtype, o, rep, st);
+    case LGF_PREC_FP64: return solve_single_any<double>(t, m, ncomp, f, phi, dtype, o, rep, st, fine);
+    case LGF_PREC_FP32: return solve_single_any<float>(t, m, ncomp, f, phi, dtype, o, rep, st, fine);
+    default: return solve_single_any<df>(t, m, ncomp, f, phi, dtype, o, rep, st, fine);
   }
 }
 

@@ -6,8 +6,9 @@ namespace lgf {
 
 Workspace *workspace_for(lgf_table *t, cudaStream_t st);
 
+// `fine`: the caller differences phi of a single level (see LineFine in lines.cuh; composite solves always run so)
 int solve_poisson(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, void *phi, int dtype,
-                  const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st);
+                  const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st, bool fine = false);
 int solve_multi(lgf_table *t, const lgf_mesh *m, int ncomp, const void *f, void *phi, int dtype,
                 const lgf_solve_opts &o, lgf_report *rep, cudaStream_t st, const lgf_indicator *ind);
 int solve_projection(lgf_table *t, const lgf_mesh *m, const void *r, void *u, void *p, int dtype, double alpha,
