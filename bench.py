@@ -159,14 +159,32 @@ def roofline(kernel, alg_bytes, kernel_ms, launches, pk, traffic=None, alg_flops
     out = {"kernel": kernel, "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
            "frac": ach / pk["hbm_gbs"], "traffic": traffic, "alg_bytes_per_step": float(alg_bytes),
            "kernel_ms_per_step": float(kernel_ms), "launches_per_step": int(launches),
-           "peak_source": pk["source"],
-           "note": "achieved = method-minimum bytes (caller fields read and written once + unique kernel-spectrum "
-                   "values, lgf_report.alg_bytes) / the kernel's CUDA-event time; " + note}
+           "peak_source": pk["source"]}
+    if note:
+        out["note"] = note
     if alg_flops is not None:
-        out["flop_view"] = {"alg_tflops": alg_flops / (kernel_ms * 1e-3) / 1e12, "alg_flops_per_step": alg_flops,
-                            "note": "5 M log2 M per complex transform (+ 8 per pair multiply-add) over the same time; "
-                                    "the double-float arithmetic runs them on the FP32 pipe"}
+        out["flop_view"] = {"alg_tflops": alg_flops / (kernel_ms * 1e-3) / 1e12, "alg_flops_per_step": alg_flops}
     return out
+
+
+ROOFLINE_NOTE = ("achieved = method-minimum bytes (caller fields read and written once + unique kernel-spectrum values, "
+                 "lgf_report.alg_bytes) / the kernel's CUDA-event time; flop_view: 5 M log2 M per complex transform (+ 8 "
+                 "per pair multiply-add) over the same time, which the double-float arithmetic runs on the FP32 pipe")
+
+
+def line_text(line):
+    """The JSON line of a result, short enough for readers that keep the end of a program's output: six significant
+    digits, and the peak only once (`peaks`, and the headline's own rooflines)."""
+    def short(v, nested):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            once = ("bound", "peak", "unit", "traffic", "peak_source") if nested and "frac" in v else ()
+            return {k: short(x, nested) for k, x in v.items() if k not in once}
+        if isinstance(v, (list, tuple)):
+            return [short(x, nested) for x in v]
+        return v
+    return json.dumps({k: short(v, isinstance(v, dict) and "frac" not in v) for k, v in line.items()})
 
 
 def flush_l2(buf):
@@ -801,9 +819,10 @@ def run_gpu(args):
             "table_build_s": hb["t_table"],
             "clocks": clocks,
             "peaks": {"hbm_gbs": pk["hbm_gbs"], "source": pk["source"]},
+            "roofline_note": ROOFLINE_NOTE,
         }
         line.update(extra)
-        print(json.dumps(line), flush=True)
+        print(line_text(line), flush=True)
     _replicas_done(world)
 
 
@@ -842,7 +861,7 @@ def run_reference(args):
                                        "oracle (dense level boxes, pocketfft convolutions)",
                              "threads_used": _oracle_threads()},
             "e2e": {"value": val, "unit": "Mcells/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    print(line_text(line), flush=True)
 
 
 def run_one(args):
@@ -894,7 +913,7 @@ def run_one(args):
                 "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "df32",
                 "data": "synthetic", "config": {"workload": name}, "detail": out, "clocks": clk.summary()}
-        print(json.dumps(line), flush=True)
+        print(line_text(line), flush=True)
     _replicas_done(world)
 
 
