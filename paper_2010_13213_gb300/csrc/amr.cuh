@@ -535,7 +535,7 @@ template <class R, int B>
 size_t heat_line_smem(int r) { return sizeof(R) * (size_t)(B + 2 * r) * (B * B + 1); }
 
 // The same pass in double-float with packed arithmetic: a thread sums a pair of adjacent lines (q = 2p, 2p + 1) as
-// f32x2 chains on (hi, hi) and (lo, lo) register pairs, the same operations as the scalar form and the same results.
+// f32x2 chains on (hi, hi) and (lo, lo) register pairs, the scalar form's operations per output.
 // The tile holds S[t][p] = (hi_2p, hi_2p+1, lo_2p, lo_2p+1).  Along y and z the pair is two neighbours in x: a thread
 // loads, sums and stores its own column (16-byte accesses); along x the tile is filled and read back in memory order.
 // Bound: the FP32 pipe (10 (2 r + 1) packed instructions per output; the scalar form issues twice as many and spent a

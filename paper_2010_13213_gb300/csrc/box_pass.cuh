@@ -1,9 +1,10 @@
 // box_pass.cuh -- block-index DFT passes of the seven-launch box convolution (direct conjugate-pair form; box_fft.cuh
 // has the in-register FFT form for 4..16 blocks), around k_box_mid.
 //
-// They serve FP32 arithmetic on FP64 fields: such callers keep single-precision results in double storage and compare
-// them digit by digit with earlier runs, so the order of the FP32 operations is kept.  Everything else runs the line
-// passes (lines.cuh), which round differently in the last bits.
+// They serve FP32 arithmetic on FP64 fields, whose results the callers read in double: the order of the FP32 operations,
+// and with it every digit beyond the sixth, is as it was before the line passes (lines.cuh), which everything else runs.
+// The interface promises about 1e-6 and no order of operations, so this is a choice, not an accuracy requirement; it costs
+// seven launches instead of five (96 x 96 x 48 ring: 108 us; FP32 fields take the line passes).
 #pragma once
 #include "box.cuh"
 

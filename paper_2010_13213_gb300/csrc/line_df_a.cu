@@ -1,4 +1,4 @@
-// Line transforms of 16 points per second step, NB = 1..6, arithmetic df.
+// Line transforms of 16 points per second step, NB = 1..6, and of 8 points, NB = 2 and 4, arithmetic df.
 #include "line_ops.cuh"
 
 namespace lgf {

@@ -32,7 +32,9 @@ const void *spectra_of<df>(const lgf_table *t) { return t->sdf; }
 
 // Relative cost model of the two ways to evaluate the per-frequency block-pair sum (complex
 // multiply-adds per real component): PAIR = nsrc * ntgt * (2B)^2 (B+1) plus the block transforms;
-// BOX = block-index DFTs over the 2 nb grid plus the local transforms, shared by two components.
+// BOX = block-index DFTs over the 2 nb grid plus the local transforms, shared by two components.  BOX counts the
+// block-index passes; the line passes (lines.cuh) take 0.55 to 0.65 of their time, so near the crossover the model favours
+// PAIR.  The crossover itself has not been measured.
 double box_cost(int B, const int nb[3]) {
   const double B3 = (double)B * B * B;
   const double nx = nb[0], ny = nb[1], nz = nb[2];
