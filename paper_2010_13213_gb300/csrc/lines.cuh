@@ -82,7 +82,7 @@ struct LineGeom {
 // lazy sums composite solves on 16^3 blocks had 1.15 times the error of the block-index passes (mean of 24 meshes, up to
 // 1.5 times) and have 0.99 times now, refreshes of a few blocks 1.28 and 1.15; plain solves have 0.81 times with lazy sums
 // and keep them.  Three-level ring 4.45 -> 4.68 ms, refresh of 6 x 6 x 3 blocks 311 -> 324 us.  Lines in 8-point steps come
-// from 8^3 blocks, where lazy sums have 0.45 to 0.85 times that error in composite solves too (5 x 7 x 3 blocks with
+// from 8^3 blocks, where lazy sums have 0.48 to 0.86 times that error in composite solves too (5 x 7 x 3 blocks with
 // renormalised sums: 36.9 -> 40.5 us).
 template <class R, int M>
 struct LineFine {
